@@ -1631,12 +1631,252 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
   finish_theta<R, D, DU, THETA>(kp, th, active, partT, red1, blockIdx.x);
 }
 
+// ---------------------------------------------------------------------------
+// Recompute adjoint with parameter gradients, where the segment's normals fit in shared
+// memory (recompute_zbuf).  The parameter gradients need every sub-step's normals and the
+// unit jump sizes, so a jump step's draws are kept once instead of being drawn again on
+// the way back.  A segment of S steps runs in four passes:
+//   draws   the main-stream words and normals of every step (normals to shared memory,
+//           one bit per step with jumps): the lanes run the same code, no state on the chain;
+//   slots   pass r draws the slot of each lane's r-th one-jump step, whatever its step, into
+//           record r (time fraction, unit sizes, the normals after the jump), so the lanes'
+//           jumps of the whole segment share one or two passes;
+//   replay  the states from the checkpoint, a one-jump step from its record;
+//   back    the adjoint; a one-jump step's post-jump state is formed again from X_k and the
+//           record (the replay's operations: the same bits).
+// Steps with several jumps and one-jump steps beyond THETA_RECS records are regenerated by
+// jump_backward.  At lambda dt = 0.01 a lane has more than two one-jump steps in 16 with
+// probability 6e-4.  Bound by instruction issue.  Before, the replay drew a jump step's slot
+// in divergent code per step and the backward regenerated every jump step through
+// jump_backward: 39.1 -> 13.8 ms per launch at M = 2^20, N_t = 1024, lambda dt = 0.0098 (27%
+// of the warp-steps have a jump).  The draws loop rolled, with the round keys from the
+// parameter block (unrolled 2 or 4 times 13.8 / 13.9 ms; keys bumped 14.1 ms).
+template <typename R, int D>
+struct ThetaRecs {
+  static constexpr int N = 2;             // records per path and segment
+  static constexpr int W = 1 + 2 * D;     // values per record
+  R *p;                                   // this thread's column
+  __device__ __forceinline__ R &at(int r, int w) const { return p[(r * W + w) * TPB]; }
+  __device__ __forceinline__ R load(int r, R (&xih)[D], R (&z1)[D]) const {
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+      xih[c] = at(r, 1 + c);
+      z1[c] = at(r, 1 + D + c);
+    }
+    return at(r, 0);
+  }
+};
+template <typename R, int D>
+__host__ __device__ constexpr size_t theta_rec_bytes() {   // per block
+  return (size_t)ThetaRecs<R, D>::N * ThetaRecs<R, D>::W * TPB * sizeof(R);
+}
+
+// One sub-step of length de (sq = sqrt(de)) from y with normals z, backwards: the noise and
+// drift-direction sensitivities, then g and mu as in the other sweeps (the operations and
+// order of jump_backward).
+template <typename R, int D, int DU>
+__device__ __forceinline__ void theta_substep(const KParams<R, D, DU> &kp, const R (&y)[D], const R (&z)[D], R de,
+                                              R sq, R (&mu)[D], R (&g)[DU], R (&th)[D + 2]) {
+  using M = Ar<R>;
+#pragma unroll
+  for (int c = 0; c < D; ++c) th[1 + c] = M::fma(M::mul(mu[c], sq), z[c], th[1 + c]);
+  if (kp.has_dA) {
+    R s = R(0);
+#pragma unroll
+    for (int r = 0; r < D; ++r)
+#pragma unroll
+      for (int c = 0; c < D; ++c) s = M::fma(M::mul(mu[r], kp.dA[r * D + c]), y[c], s);
+    th[0] = M::fma(de, s, th[0]);
+  }
+  control_sensitivity(kp, mu, de, g);
+  adjoint_update(kp, y, de, mu);
+}
+
+template <typename R, int D, int DU>
+__device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, const R *__restrict__ u,
+                                               const R *__restrict__ xd, const R *__restrict__ ckpt,
+                                               double *__restrict__ partG, double *__restrict__ partT,
+                                               int64_t mloc) {
+  using M = Ar<R>;
+  constexpr int CH = 8, NR = 8;
+  extern __shared__ __align__(16) unsigned char dsm[];
+  R *sbuf = reinterpret_cast<R *>(dsm);   // [S * D][TPB] segment states
+  const int S = kp.S;
+  R *zbuf = sbuf + (size_t)S * D * TPB;   // [S * D][TPB] main-stream normals
+  const int tid = threadIdx.x;
+  const ThetaRecs<R, D> rec{zbuf + (size_t)S * D * TPB + tid};   // [N * W][TPB]
+  GradRows<R, DU, NR> rows;
+  rows.init(zbuf + (size_t)S * D * TPB + ThetaRecs<R, D>::N * ThetaRecs<R, D>::W * TPB);
+  __shared__ Pair<R> red1[TPB / 32];
+  const int64_t npart = kp.npart;
+  const int64_t lm = (int64_t)blockIdx.x * TPB + tid;
+  const bool active = lm < mloc;
+  const int64_t lmc = active ? lm : 0;   // inactive threads replay path 0
+  const uint32_t m = (uint32_t)(kp.m_begin + lmc);
+  const int Nt = kp.Nt;
+  const int nseg = (Nt + S - 1) / S;
+  R mu[D], th[D + 2];
+#pragma unroll
+  for (int t = 0; t < D + 2; ++t) th[t] = R(0);
+  {
+    R xN[D];
+    load_row<R, D>(xd + (size_t)Nt * D, xN);
+#pragma unroll
+    for (int c = 0; c < D; ++c)
+      mu[c] = M::mul(kp.qdt[c], M::sub(__ldg(ckpt + ((size_t)nseg * D + c) * mloc + lmc), xN[c]));
+  }
+#pragma unroll 1
+  for (int seg = nseg - 1; seg >= 0; --seg) {
+    const int k0 = seg * S, len = min(S, Nt - k0);
+    R x[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) x[c] = __ldg(ckpt + ((size_t)seg * D + c) * mloc + lmc);
+    // bit i: step k0 + i had jumps (jm); exactly one (om) (S <= 64)
+    uint64_t jm = 0, om = 0;
+#pragma unroll 1
+    for (int i = 0; i < len; ++i) {
+      R z[D];
+      const uint32_t w0 = main_draws<true>(kp, k0 + i, m, z);
+#pragma unroll
+      for (int c = 0; c < D; ++c) zbuf[(i * D + c) * TPB + tid] = z[c];
+      if (has_jump(kp, w0)) {
+        jm |= 1ull << i;
+        if (one_jump(kp, w0)) om |= 1ull << i;
+      }
+    }
+    uint64_t rm = 0;   // steps with a record, in record order
+#pragma unroll 1
+    for (int r = 0; r < ThetaRecs<R, D>::N; ++r) {
+      if (om == 0) continue;
+      const int i = __ffsll((long long)om) - 1;
+      om &= om - 1;
+      rm |= 1ull << i;
+      R xih[D], z1[D];
+      rec.at(r, 0) = slot0_draws<true>(kp, k0 + i, m, xih, z1);
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        rec.at(r, 1 + c) = xih[c];
+        rec.at(r, 1 + D + c) = z1[c];
+      }
+    }
+    int rr = 0;
+#pragma unroll 1
+    for (int i = 0; i < len; ++i) {
+      const int k = k0 + i;
+      R z[D], uk[DU];
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        sbuf[(i * D + c) * TPB + tid] = x[c];
+        z[c] = zbuf[(i * D + c) * TPB + tid];
+      }
+#pragma unroll
+      for (int l = 0; l < DU; ++l) uk[l] = __ldg(u + (size_t)k * DU + l);
+      if (!((jm >> i) & 1u)) {
+        R f[D];
+        drift(kp, x, uk, f);
+        plain_update(kp, f, z, x);
+      } else if ((rm >> i) & 1u) {
+        R xih[D], z1[D];
+        const R t1 = rec.load(rr++, xih, z1);
+        euler_substep(kp, M::mul(kp.dt, t1), z, uk, x);
+        apply_jump(kp, x, xih);
+        euler_substep(kp, M::mul(kp.dt, M::sub(R(1), t1)), z1, uk, x);
+      } else {   // several jumps, or no record left: the general routine, on copies
+        JumpStep<R, D> js;
+        R xl[D], ul[DU];
+#pragma unroll
+        for (int c = 0; c < D; ++c) xl[c] = x[c];
+#pragma unroll
+        for (int l = 0; l < DU; ++l) ul[l] = uk[l];
+        R zl[D];
+        const uint32_t w0 = main_draws(kp, k, m, zl);
+        build_jump_step(kp, k, m, w0, zl, ul, xl, &js);
+#pragma unroll
+        for (int c = 0; c < D; ++c) x[c] = js.Y[js.n + 1][c];
+      }
+    }
+    const int nch = (len + CH - 1) / CH;
+#pragma unroll 1
+    for (int cc = nch - 1; cc >= 0; --cc) {
+      const int i0 = cc * CH;
+#pragma unroll 1
+      for (int j = CH - 1; j >= 0; --j) {
+        const int i = i0 + j, k = k0 + i;
+        R g[DU];
+#pragma unroll
+        for (int l = 0; l < DU; ++l) g[l] = R(0);
+        if (i < len) {
+          R xk[D], z[D];
+#pragma unroll
+          for (int c = 0; c < D; ++c) {
+            xk[c] = sbuf[(i * D + c) * TPB + tid];
+            z[c] = zbuf[(i * D + c) * TPB + tid];
+          }
+          if (!((jm >> i) & 1u)) {
+            theta_substep(kp, xk, z, kp.dt, kp.sqdt, mu, g, th);
+          } else if ((rm >> i) & 1u) {
+            R xih[D], z1[D], y[D], uk[DU];
+            const R t1 = rec.load(--rr, xih, z1);
+#pragma unroll
+            for (int l = 0; l < DU; ++l) uk[l] = __ldg(u + (size_t)k * DU + l);
+            const R de0 = M::mul(kp.dt, t1), de1 = M::mul(kp.dt, M::sub(R(1), t1));
+#pragma unroll
+            for (int c = 0; c < D; ++c) y[c] = xk[c];
+            euler_substep(kp, de0, z, uk, y);
+            apply_jump(kp, y, xih);
+            theta_substep(kp, y, z1, de1, M::sqrt(de1), mu, g, th);
+            R s = R(0);   // d/d jump_scale: the components the jump moves
+#pragma unroll
+            for (int c = 0; c < D; ++c)
+              if (c >= kp.kvel) s = M::fma(mu[c], xih[c], s);
+            th[D + 1] = M::add(th[D + 1], s);
+            if (kp.jump_law == JD_JUMP_KS) jump_adjoint(kp, mu);
+            theta_substep(kp, xk, z, de0, M::sqrt(de0), mu, g, th);
+          } else {
+            R xl[D], ml[D], gl[DU], tl[D + 2], ul[DU];
+#pragma unroll
+            for (int c = 0; c < D; ++c) {
+              xl[c] = xk[c];
+              ml[c] = mu[c];
+            }
+#pragma unroll
+            for (int l = 0; l < DU; ++l) {
+              gl[l] = R(0);
+              ul[l] = __ldg(u + (size_t)k * DU + l);
+            }
+#pragma unroll
+            for (int t = 0; t < D + 2; ++t) tl[t] = th[t];
+            jump_backward<R, D, DU, true>(kp, k, m, xl, ul, ml, gl, tl);
+#pragma unroll
+            for (int c = 0; c < D; ++c) mu[c] = ml[c];
+#pragma unroll
+            for (int l = 0; l < DU; ++l) g[l] = gl[l];
+#pragma unroll
+            for (int t = 0; t < D + 2; ++t) th[t] = tl[t];
+          }
+          if (k >= 1) {
+            R xdk[D];
+            load_row<R, D>(xd + (size_t)k * D, xdk);
+            cost_gradient(kp, xk, xdk, mu);
+          }
+        }
+        rows.put(k & (NR - 1), g, active);
+      }
+      if (((k0 + i0) & (NR - 1)) == 0) rows.flush(k0 + i0, Nt, partG, npart, blockIdx.x);
+    }
+  }
+  finish_theta<R, D, DU, true>(kp, th, active, partT, red1, blockIdx.x);
+}
+
 template <typename R, int D, int DU, bool THETA>
 __global__ void __launch_bounds__(TPB)
 adj_recompute_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u,
                      const R *__restrict__ xd, const R *__restrict__ ckpt,
                      double *__restrict__ partG, double *__restrict__ partT, int64_t mloc) {
-  adj_recompute_body<R, D, DU, THETA>(kp, u, xd, ckpt, partG, partT, mloc);
+  if constexpr (THETA && recompute_zbuf<R, D, THETA>())
+    adj_theta_body<R, D, DU>(kp, u, xd, ckpt, partG, partT, mloc);
+  else
+    adj_recompute_body<R, D, DU, THETA>(kp, u, xd, ckpt, partG, partT, mloc);
 }
 
 // The parameter-gradient form for FP32 d <= 2 with at least 5 blocks per SM: the default
@@ -1647,7 +1887,7 @@ __global__ void __launch_bounds__(TPB, 5)
 adj_recompute_theta5_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u,
                             const R *__restrict__ xd, const R *__restrict__ ckpt,
                             double *__restrict__ partG, double *__restrict__ partT, int64_t mloc) {
-  adj_recompute_body<R, D, DU, true>(kp, u, xd, ckpt, partG, partT, mloc);
+  adj_theta_body<R, D, DU>(kp, u, xd, ckpt, partG, partT, mloc);
 }
 
 template <typename R, int D>
@@ -1854,7 +2094,8 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
 // Shared memory of the recompute adjoint for segments of S steps.
 template <typename R, int D, int DU>
 size_t recompute_smem(bool theta, int S) {
-  return (size_t)S * D * TPB * sizeof(R) * (theta && recompute_zbuf<R, D, true>() ? 2 : 1) +
+  const bool zbuf = theta && recompute_zbuf<R, D, true>();
+  return (size_t)S * D * TPB * sizeof(R) * (zbuf ? 2 : 1) + (zbuf ? theta_rec_bytes<R, D>() : 0) +
          (theta ? 0 : (size_t)seg_log_cap<D>() * (2 + D) * TPB * sizeof(R)) + grad_rows_bytes<R, DU, 8>();
 }
 
