@@ -45,6 +45,7 @@ struct KParams {
   // sweeps as constant operands of the rounds' XORs instead of bumping the key in every
   // block; last in the struct, so kernels that do not read them see the same layout
   uint32_t rk0[10], rk1[10];
+  int chunk;                      // steps per chunk of the chunked forward sweep (4, 8 or 16)
 };
 
 // Device buffers of one launch (unused ones are null).

@@ -255,10 +255,32 @@ __host__ __device__ constexpr int seg_len() {
 }
 
 // Steps with one jump take a short path (the common case); two or more go through
-// build_jump_step.  The jump map (apply_jump) covers every law on both paths: with the
-// additive laws jgain = 1, so y + s xih bit for bit.  (Keilson-Storer steps all went through
-// build_jump_step before: 5.26 -> 4.13 ms per store sweep at M = 2^20, N_t = 500, lambda dt =
-// 0.0036, where 11% of the warp-steps have a jump.)
+// build_jump_step.  The short path takes every law for d <= 2 (Keilson-Storer steps all went
+// through build_jump_step before: 5.26 -> 4.13 ms per store sweep at M = 2^20, N_t = 500,
+// lambda dt = 0.0036, where 11% of the warp-steps have a jump), the additive laws for larger
+// d (whose sweeps ran 1% slower with the law's branch).
+template <int D>
+constexpr bool ONE_JUMP_KS = D <= 2;
+// The step has exactly one jump and its slot words lie as compiled (the one-jump paths).
+template <typename R, int D, int DU>
+__device__ __forceinline__ bool one_jump(const KParams<R, D, DU> &kp, uint32_t w0) {
+  return (ONE_JUMP_KS<D> || kp.jump_law != JD_JUMP_KS) && kp.npair == MainWords<D>::PD &&
+         (unsigned long long)w0 < kp.thr[1];
+}
+
+// The jump of a one-jump step (apply_jump; the additive map without its product by jgain = 1,
+// the same bits).
+template <typename R, int D, int DU>
+__device__ __forceinline__ void apply_one_jump(const KParams<R, D, DU> &kp, R (&x)[D], const R (&xih)[D]) {
+  using M = Ar<R>;
+  if (ONE_JUMP_KS<D> && kp.jump_law == JD_JUMP_KS) {
+    apply_jump(kp, x, xih);
+  } else {
+#pragma unroll
+    for (int c = 0; c < D; ++c) x[c] = M::add(x[c], M::mul(kp.jump_scale, xih[c]));
+  }
+}
+
 // The one-jump step out of line: sub-step to the jump, jump, sub-step to t_{k+1}.  x is
 // updated in place; y1 receives the post-jump state; returns the jump's time fraction.
 template <typename R, int D, int DU>
@@ -275,19 +297,13 @@ __device__ __noinline__ R one_jump_substeps(const KParams<R, D, DU> &kp, int k, 
   for (int l = 0; l < DU; ++l) ul[l] = uk[l];
   const R th = slot0_draws(kp, k, m, xih, z1);
   euler_substep(kp, M::mul(kp.dt, th), zz, ul, xl);
-  apply_jump(kp, xl, xih);
+  apply_one_jump(kp, xl, xih);
 #pragma unroll
   for (int c = 0; c < D; ++c) y1[c] = xl[c];
   euler_substep(kp, M::mul(kp.dt, M::sub(R(1), th)), z1, ul, xl);
 #pragma unroll
   for (int c = 0; c < D; ++c) x[c] = xl[c];
   return th;
-}
-
-// The step has exactly one jump and its slot words lie as compiled (the one-jump paths).
-template <typename R, int D, int DU>
-__device__ __forceinline__ bool one_jump(const KParams<R, D, DU> &kp, uint32_t w0) {
-  return kp.npair == MainWords<D>::PD && (unsigned long long)w0 < kp.thr[1];
 }
 
 // The one-jump step inline, its slot draws (time fraction th, jump size xih, second
@@ -298,14 +314,7 @@ __device__ __forceinline__ void one_jump_inline(const KParams<R, D, DU> &kp, int
                                                 LW &lw) {
   using M = Ar<R>;
   euler_substep(kp, M::mul(kp.dt, th), z, uk, x);
-  // the additive map without its product by jgain = 1 (the same bits): eight fewer
-  // products per jump at d = 8
-  if (D > 2 && kp.jump_law != JD_JUMP_KS) {
-#pragma unroll
-    for (int c = 0; c < D; ++c) x[c] = M::add(x[c], M::mul(kp.jump_scale, xih[c]));
-  } else {
-    apply_jump(kp, x, xih);
-  }
+  apply_one_jump(kp, x, xih);
   if constexpr (!std::is_same<LW, NoLog>::value) {
     if (lw.take(1, k)) lw.put(k, 0, th, x);
   }
@@ -325,6 +334,23 @@ __device__ __forceinline__ void plain_update(const KP &kp, const R (&f)[D], cons
       }
     } else {
       x[c] = M::fma(kp.sig_sqdt[c], z[c], M::fma(kp.dt, f[c], x[c]));
+    }
+  }
+}
+
+// x <- x + de f + a z (a = sigma sqrt(de)): a sub-step whose noise scale is given.
+template <typename R, int D>
+__device__ __forceinline__ void noisy_update(R de, const R (&f)[D], const R (&a)[D], const R (&z)[D], R (&x)[D]) {
+  using M = Ar<R>;
+#pragma unroll
+  for (int c = 0; c < D; ++c) {
+    if constexpr (Pr<R>::on && D % 2 == 0) {
+      if (c % 2 == 0) {
+        Pr<R>::fma(de, de, f[c], f[c + 1], x[c], x[c + 1]);
+        Pr<R>::fma(a[c], a[c + 1], z[c], z[c + 1], x[c], x[c + 1]);
+      }
+    } else {
+      x[c] = M::fma(a[c], z[c], M::fma(de, f[c], x[c]));
     }
   }
 }
@@ -462,9 +488,36 @@ __device__ __forceinline__ int forward_step2(const KParams<R, D, DU> &kp, const 
   return n;
 }
 
+// Target row x_d(t_k): D values, as vector loads where the row's size and alignment allow.
+template <typename R, int D>
+__device__ __forceinline__ void load_row(const R *__restrict__ p, R (&o)[D]) {
+  if constexpr (sizeof(R) == 4 && D % 4 == 0) {
+#pragma unroll
+    for (int c = 0; c < D; c += 4) {
+      const float4 v = __ldg(reinterpret_cast<const float4 *>(p + c));
+      o[c] = v.x; o[c + 1] = v.y; o[c + 2] = v.z; o[c + 3] = v.w;
+    }
+  } else if constexpr (sizeof(R) == 4 && D % 2 == 0) {
+#pragma unroll
+    for (int c = 0; c < D; c += 2) {
+      const float2 v = __ldg(reinterpret_cast<const float2 *>(p + c));
+      o[c] = v.x; o[c + 1] = v.y;
+    }
+  } else if constexpr (sizeof(R) == 8 && D % 2 == 0) {
+#pragma unroll
+    for (int c = 0; c < D; c += 2) {
+      const double2 v = __ldg(reinterpret_cast<const double2 *>(p + c));
+      o[c] = v.x; o[c + 1] = v.y;
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < D; ++c) o[c] = __ldg(p + c);
+  }
+}
+
 // dt l(x, t_k) = sum_c (q_c dt / 2) (x_c - xd_c(t_k))^2
 template <typename KP, typename R, int D>
-__device__ __forceinline__ R cost_term(const KP &kp, const R (&x)[D], const R *__restrict__ xdk) {
+__device__ __forceinline__ R cost_term_row(const KP &kp, const R (&x)[D], const R (&xdk)[D]) {
   using M = Ar<R>;
   R t = R(0);
   if constexpr (Pr<R>::on && D % 2 == 0) {
@@ -472,7 +525,7 @@ __device__ __forceinline__ R cost_term(const KP &kp, const R (&x)[D], const R *_
 #pragma unroll
     for (int c = 0; c < D; c += 2) {
       R e0, e1, h0, h1;
-      Pr<R>::sub(x[c], x[c + 1], __ldg(xdk + c), __ldg(xdk + c + 1), e0, e1);
+      Pr<R>::sub(x[c], x[c + 1], xdk[c], xdk[c + 1], e0, e1);
       Pr<R>::mul(kp.hqdt[c], kp.hqdt[c + 1], e0, e1, h0, h1);
       t = M::fma(h0, e0, t);
       t = M::fma(h1, e1, t);
@@ -481,10 +534,232 @@ __device__ __forceinline__ R cost_term(const KP &kp, const R (&x)[D], const R *_
   }
 #pragma unroll
   for (int c = 0; c < D; ++c) {
-    const R e = M::sub(x[c], __ldg(xdk + c));
+    const R e = M::sub(x[c], xdk[c]);
     t = M::fma(M::mul(kp.hqdt[c], e), e, t);
   }
   return t;
+}
+
+template <typename KP, typename R, int D>
+__device__ __forceinline__ R cost_term(const KP &kp, const R (&x)[D], const R *__restrict__ xdk) {
+  R row[D];
+#pragma unroll
+  for (int c = 0; c < D; ++c) row[c] = __ldg(xdk + c);
+  return cost_term_row(kp, x, row);
+}
+
+// ---------------------------------------------------------------------------
+// Forward steps of d <= 2 in chunks.  A step with jumps costs its warp a pass of divergent
+// code for every lane that jumps; most of that pass is the slot's draws, which depend on
+// nothing but the counters.  A chunk of steps therefore runs in three passes:
+//   draws   the main-stream words and normals of every step (normals to shared memory, the
+//           jump decisions to bit masks), the lanes in step and no state on the chain;
+//   slots   pass r draws each lane's r-th jump of the chunk, whichever step it lies in, into
+//           record r, with the square roots of a one-jump step's sub-steps: the lanes' jumps
+//           of the whole chunk share one or two passes;
+//   steps   the states, the running cost and the stores; a step with one or two jumps takes
+//           its records, any other jump step the general routine.
+// The draws and the arithmetic of every step are step_from_draws', so the same bits.
+// ---------------------------------------------------------------------------
+template <int D>
+constexpr bool fwd_chunked() {
+  return D <= 2;
+}
+template <typename R, int D>
+struct FwdChunk {
+  static constexpr int CH = sizeof(R) * D <= 8 ? 16 : 8;   // steps per chunk at most
+  // record: time fraction, jscl xih, normals after the jump; a step with one jump also has
+  // the noise scales sigma sqrt(delta) of its two sub-steps
+  static constexpr int TH = 0, XJ = 1, Z1 = 1 + D, A0 = 1 + 2 * D, A1 = 1 + 3 * D, W = 1 + 4 * D;
+};
+// Chunk length: the records hold a lane's jumps of a chunk but in rare chunks, and a pass of
+// slot draws serves many lanes.
+inline int fwd_chunk_len(double lamdt, int most) {
+  const int n = lamdt <= 0.015 ? 16 : lamdt <= 0.03 ? 8 : 4;
+  return n < most ? n : most;
+}
+
+// Whether a sweep takes its steps in chunks, by the jump rate per step.  The store sweep and
+// every FP64 sweep gain or tie at any rate; the other FP32 sweeps pay about 6% for the
+// chunks' passes without jumps and gain from about lambda dt = 0.005 on.  One launch at M =
+// 2^20, N_t = 160, d = 2 FP32, step by step -> in chunks, in ms:
+//   lambda dt          0            0.002         0.01          0.05          0.2           0.4
+//   cost          0.91 -> 0.97  1.01 -> 1.06  1.32 -> 1.23  2.33 -> 1.94  5.88 -> 3.27  9.96 -> 7.08
+//   store         1.11 -> 1.04  1.21 -> 1.15  1.56 -> 1.38  2.66 -> 2.24  6.38 -> 3.83  10.5 -> 8.48
+//   checkpoints   0.94 -> 0.99  1.02 -> 1.09  1.32 -> 1.25  2.30 -> 1.97  5.97 -> 3.34  10.1 -> 7.55
+//   store, pair   1.25 -> 1.22  1.38 -> 1.39  1.82 -> 1.79  4.16 -> 3.03  12.9 -> 6.65  21.9 -> 15.7
+//   ckpt., pair   1.11 -> 1.15  1.21 -> 1.27  1.59 -> 1.51  3.16 -> 2.44  10.1 -> 4.69  18.4 -> 11.9
+//   recompute     1.26 -> 1.35  1.39 -> 1.47  1.80 -> 1.70  3.18 -> 2.75  12.1 -> 12.1  23.7 -> 22.1
+//   adjoint (replay)
+// (double precision, M = 2^15: store sweep 1.17 -> 1.17, 1.30 -> 1.28, 1.68 -> 1.49, 2.68 ->
+// 2.17, 4.32 -> 4.14 ms up to 0.2.)  Between 0.004 and 0.007 the forms are within 3%.
+constexpr double FWD_CHUNK_RATE = 0.006;
+template <typename R, int D>
+inline bool fwd_chunks(double lamdt, bool single_store) {
+  return fwd_chunked<D>() && (sizeof(R) == 8 || single_store || lamdt > FWD_CHUNK_RATE);
+}
+
+// Bits of a chunk, bit i for its step i: jumps; two or more; the jumps have records (in
+// record order); some lane of the warp jumps (warp-uniform: the steps pass runs a step in
+// which no lane jumps without a test per lane).
+struct ChunkBits {
+  uint32_t jump, two, rec, any;
+  __device__ __forceinline__ int records(int i) const {
+    return ((rec >> i) & 1u) ? 1 + (int)((two >> i) & 1u) : 0;
+  }
+};
+
+// Normals of chunk step i in this thread's column: d = 2 as one vector of two values.
+template <typename R, int D>
+__device__ __forceinline__ void put_normals(R (*z)[TPB], int i, const R (&v)[D]) {
+  if constexpr (D == 2)
+    reinterpret_cast<typename V2<R>::T *>(z[2 * i])[threadIdx.x] = V2<R>::make(v[0], v[1]);
+  else
+    z[i][threadIdx.x] = v[0];
+}
+template <typename R, int D>
+__device__ __forceinline__ void get_normals(const R (*z)[TPB], int i, R (&v)[D]) {
+  if constexpr (D == 2) {
+    const typename V2<R>::T t = reinterpret_cast<const typename V2<R>::T *>(z[2 * i])[threadIdx.x];
+    v[0] = t.x;
+    v[1] = t.y;
+  } else {
+    v[0] = z[i][threadIdx.x];
+  }
+}
+
+// The draws and slots passes of the len steps from k0: the normals of step i go to rows
+// i D .. i D + D - 1 of z (put_normals), up to nrec records of W rows to rec (this thread's column).
+template <typename R, int D, int DU, int UNR, bool RK>
+__device__ __forceinline__ ChunkBits chunk_draws(const KParams<R, D, DU> &kp, int k0, int len, uint32_t m,
+                                                 R (*z)[TPB], R (*rec)[TPB], int nrec) {
+  using M = Ar<R>;
+  using F = FwdChunk<R, D>;
+  const int tid = threadIdx.x;
+  ChunkBits b{0, 0, 0, 0};
+  // 32-bit thresholds; a count that cannot be reached (threshold 2^32) is masked at the end
+  const uint32_t t1 = (uint32_t)min(kp.thr[0], 0xffffffffull), t2 = (uint32_t)min(kp.thr[1], 0xffffffffull);
+  const uint32_t t3 = (uint32_t)min(kp.thr[2], 0xffffffffull);
+  uint32_t bit = 1, three = 0;
+#pragma unroll UNR
+  for (int i = 0; i < len; ++i, bit += bit) {
+    R zi[D];
+    const uint32_t w0 = main_draws<RK>(kp, k0 + i, m, zi);
+    put_normals<R, D>(z, i, zi);
+    b.jump |= w0 >= t1 ? bit : 0u;
+    b.two |= w0 >= t2 ? bit : 0u;
+    three |= w0 >= t3 ? bit : 0u;
+  }
+  b.jump &= kp.jumps_on && kp.thr[0] <= 0xffffffffull ? ~0u : 0u;
+  b.two &= kp.jumps_on && kp.thr[1] <= 0xffffffffull ? ~0u : 0u;
+  b.any = __reduce_or_sync(0xffffffffu, b.jump);
+  uint32_t pend = kp.npair == MainWords<D>::PD ? b.jump : 0u;
+  pend &= kp.thr[2] <= 0xffffffffull ? ~three : ~0u;
+  int sl = 0;
+#pragma unroll 1
+  for (int r = 0; r < nrec && pend != 0u; ++r, rec += F::W) {
+    const int i = __ffs((int)pend) - 1;
+    const bool first_of_two = ((b.two >> i) & 1u) && sl == 0;
+    if (first_of_two && r + 2 > nrec) break;
+    R xih[D], z1[D];
+    const R th = slot_draws_at<RK>(kp, k0 + i, m, sl, xih, z1);
+    const R sq0 = M::sqrt(M::mul(kp.dt, th)), sq1 = M::sqrt(M::mul(kp.dt, M::sub(R(1), th)));
+    rec[F::TH][tid] = th;
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+      rec[F::XJ + c][tid] = M::mul(kp.jscl[c], xih[c]);
+      rec[F::Z1 + c][tid] = z1[c];
+      rec[F::A0 + c][tid] = M::mul(kp.sigma[c], sq0);
+      rec[F::A1 + c][tid] = M::mul(kp.sigma[c], sq1);
+    }
+    sl = first_of_two ? 1 : 0;
+    if (!first_of_two) {
+      b.rec |= 1u << i;
+      pend &= pend - 1u;
+    }
+  }
+  return b;
+}
+
+// One step of the steps pass in which some lane of the warp jumps: the state x of one
+// control at step k with the step's normals z; jumped: this lane jumps; nrec: its records,
+// the first at rec (0 with jumped: the general routine).
+template <typename R, int D, int DU, typename LW, typename KH>
+__device__ __forceinline__ void chunk_step(const KParams<R, D, DU> &kp, const KH &kh, int k, uint32_t m, bool jumped,
+                                           int nrec, const R (*rec)[TPB], const R (&z)[D], const R (&uk)[DU],
+                                           R (&x)[D], LW &lw) {
+  using M = Ar<R>;
+  using F = FwdChunk<R, D>;
+  constexpr bool LOG = !std::is_same<LW, NoLog>::value;
+  const int tid = threadIdx.x;
+  if (!jumped) {
+    R f[D];
+    drift(kh, x, uk, f);
+    plain_update(kh, f, z, x);
+  } else if (nrec == 1) {
+    const R th = rec[F::TH][tid];
+    R a[D], zn[D], f[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) a[c] = rec[F::A0 + c][tid];
+    drift(kh, x, uk, f);
+    noisy_update(M::mul(kh.dt, th), f, a, z, x);
+#pragma unroll
+    for (int c = 0; c < D; ++c) {
+      x[c] = M::add(M::mul(kp.jgain[c], x[c]), rec[F::XJ + c][tid]);
+      a[c] = rec[F::A1 + c][tid];
+      zn[c] = rec[F::Z1 + c][tid];
+    }
+    if constexpr (LOG) {
+      if (lw.take(1, k)) lw.put(k, 0, th, x);
+    }
+    drift(kh, x, uk, f);
+    noisy_update(M::mul(kh.dt, M::sub(R(1), th)), f, a, zn, x);
+  } else if (nrec == 2) {
+    bool log = false;
+    if constexpr (LOG) log = lw.take(2, k);
+    // in time order, slot 0 first when the times are equal
+    const int swap = rec[F::TH][tid] > rec[F::W + F::TH][tid] ? 1 : 0;
+    R prev = R(0), zc[D];
+#pragma unroll
+    for (int c = 0; c < D; ++c) zc[c] = z[c];
+#pragma unroll 1
+    for (int e = 0; e <= 2; ++e) {
+      const R(*const re)[TPB] = rec + (min(e, 1) ^ swap) * F::W;
+      const R th = e < 2 ? re[F::TH][tid] : R(1);
+      euler_substep(kp, M::mul(kp.dt, M::sub(th, prev)), zc, uk, x);
+      if (e == 2) break;
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        x[c] = M::add(M::mul(kp.jgain[c], x[c]), re[F::XJ + c][tid]);
+        zc[c] = re[F::Z1 + c][tid];
+      }
+      if constexpr (LOG) {
+        if (log) lw.put(k, e, th, x);
+      }
+      prev = th;
+    }
+  } else {   // the general routine, on copies
+    JumpStep<R, D> S;
+    R xl[D], zl[D], ul[DU];
+    const uint32_t w0 = main_draws(kp, k, m, zl);
+#pragma unroll
+    for (int c = 0; c < D; ++c) xl[c] = x[c];
+#pragma unroll
+    for (int l = 0; l < DU; ++l) ul[l] = uk[l];
+    build_jump_step(kp, k, m, w0, zl, ul, xl, &S);
+#pragma unroll
+    for (int c = 0; c < D; ++c) x[c] = S.Y[S.n + 1][c];
+    if constexpr (LOG) {
+      if (lw.take(S.n, k)) {
+        for (int e = 0; e < S.n; ++e) {
+          R y[D];
+#pragma unroll
+          for (int c = 0; c < D; ++c) y[c] = S.Y[e + 1][c];
+          lw.put(k, e, S.th[e], y);
+        }
+      }
+    }
+  }
 }
 
 // Backward through a step that had jumps: regenerate its draws and sub-states from
@@ -740,33 +1015,6 @@ __device__ __forceinline__ void backward_step(const KParams<R, D, DU> &kp, const
       for (int c = 0; c < D; ++c)
         mu[c] = M::fma(kh.qdt[c], M::sub(xk[c], __ldg(xd + (size_t)k * D + c)), mu[c]);
     }
-  }
-}
-
-// Target row x_d(t_k): D values, as vector loads where the row's size and alignment allow.
-template <typename R, int D>
-__device__ __forceinline__ void load_row(const R *__restrict__ p, R (&o)[D]) {
-  if constexpr (sizeof(R) == 4 && D % 4 == 0) {
-#pragma unroll
-    for (int c = 0; c < D; c += 4) {
-      const float4 v = __ldg(reinterpret_cast<const float4 *>(p + c));
-      o[c] = v.x; o[c + 1] = v.y; o[c + 2] = v.z; o[c + 3] = v.w;
-    }
-  } else if constexpr (sizeof(R) == 4 && D % 2 == 0) {
-#pragma unroll
-    for (int c = 0; c < D; c += 2) {
-      const float2 v = __ldg(reinterpret_cast<const float2 *>(p + c));
-      o[c] = v.x; o[c + 1] = v.y;
-    }
-  } else if constexpr (sizeof(R) == 8 && D % 2 == 0) {
-#pragma unroll
-    for (int c = 0; c < D; c += 2) {
-      const double2 v = __ldg(reinterpret_cast<const double2 *>(p + c));
-      o[c] = v.x; o[c + 1] = v.y;
-    }
-  } else {
-#pragma unroll
-    for (int c = 0; c < D; ++c) o[c] = __ldg(p + c);
   }
 }
 
@@ -1163,6 +1411,182 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
   }
 }
 
+// The chunked forward sweep of block bid (the launch forms of fwd_body without PRE).  Bound
+// by instruction issue: M = 2^20, N_t = 1000, lambda dt = 0.01 (double well), store sweep
+// 9.60 -> 8.57 ms.  Without jumps a step of the cost sweep takes 1.9 ms of Philox rounds, 2.1
+// of the Box-Muller transform and 1.7 of the rest (parts of the sweep left out, per 1000
+// steps); the jumps, 2.5 ms before, take about 1.5.  Records per path and chunk and the draws
+// loop's unrolling, measured: single sweeps 2 records (64 registers; 3: 72 and 1% slower),
+// unrolled twice (1% faster); the paired sweep 3 records, rolled (unrolled 15% slower).
+template <typename R, int D, bool PAIR>
+struct __align__(16) FwdChunkSmem {
+  static constexpr int ROWS = FwdChunk<R, D>::CH * D + (PAIR ? 3 : 2) * FwdChunk<R, D>::W;
+  R row[ROWS][TPB];   // a chunk's normals, then its records (a shorter chunk leaves room for more)
+};
+
+// One group of SV states of a path as its 16-byte vectors.
+template <typename R, int D>
+__device__ __forceinline__ void store_group(R *__restrict__ traj, int g, int64_t mloc, int64_t lm,
+                                            const R (&b)[TS<R, D>::SV][D]) {
+  constexpr int VD = TS<R, D>::VD, VW = TS<R, D>::VW;
+#pragma unroll
+  for (int v = 0; v < VD; ++v) {
+    R o[VW];
+#pragma unroll
+    for (int w = 0; w < VW; ++w) o[w] = b[(v * VW + w) / D][(v * VW + w) % D];
+    Vec16<R>::store(traj + (((size_t)g * VD + v) * mloc + lm) * VW, o);
+  }
+}
+
+template <typename R, int D, int DU, int MODE, bool PAIR, bool RK, int UNR>
+__device__ __forceinline__ void fwd_chunk_body(const KParams<R, D, DU> &kp, int64_t bid, const R *__restrict__ u,
+                                               const R *__restrict__ xd, double *__restrict__ partC,
+                                               R *__restrict__ traj, uint32_t *__restrict__ flags,
+                                               R *__restrict__ ckpt, R *__restrict__ pcost, const JLog<R, D> &jl,
+                                               int *__restrict__ jcnt, int64_t mloc, const PairOut<R, D> &p2,
+                                               FwdChunkSmem<R, D, PAIR> &sm, Pair<R> *red) {
+  using M = Ar<R>;
+  constexpr int SV = TS<R, D>::SV, NC = PAIR ? 2 : 1;
+  static_assert(FwdChunk<R, D>::CH % SV == 0 && 4 % SV == 0, "chunks hold whole store groups");
+  const int tid = threadIdx.x;
+  const int64_t lm = bid * TPB + tid;
+  const bool active = lm < mloc;
+  const uint32_t m = (uint32_t)(kp.m_begin + lm);
+  const int Nt = kp.Nt, L = kp.chunk;
+  R x[NC][D];
+#pragma unroll
+  for (int h = 0; h < NC; ++h)
+#pragma unroll
+    for (int c = 0; c < D; ++c) x[h][c] = kp.x0[c];
+  Kahan<R> cost[NC];
+  uint32_t fw = 0;
+  using LW = typename std::conditional<MODE == FWD_STORE, LogWriter<R, D>, NoLog>::type;
+  LW lw[NC];
+  if constexpr (MODE == FWD_STORE) {
+#pragma unroll
+    for (int h = 0; h < NC; ++h) {
+      lw[h].L = h ? p2.jl : jl;
+      lw[h].idx = lm;
+      if (!active) lw[h].L.cap = 0;   // inactive threads log nothing
+    }
+  }
+  const HotFwd<R, D, DU> kh = hot_fwd(kp);
+  R buf[NC][SV][D];   // store mode: the states of the current group
+  R(*const rec)[TPB] = sm.row + L * D;
+  const int nrec = (FwdChunkSmem<R, D, PAIR>::ROWS - L * D) / FwdChunk<R, D>::W;
+#pragma unroll 1
+  for (int k0 = 0; k0 < Nt; k0 += L) {
+    const int len = min(L, Nt - k0);
+    if (MODE == FWD_CKPT && active && (k0 & (kp.S - 1)) == 0) {   // S is a multiple of the chunk
+#pragma unroll
+      for (int h = 0; h < NC; ++h)
+#pragma unroll
+        for (int c = 0; c < D; ++c) (h ? p2.ckpt : ckpt)[((size_t)(k0 / kp.S) * D + c) * mloc + lm] = x[h][c];
+    }
+    const ChunkBits cb =
+        chunk_draws<R, D, DU, UNR, RK>(kp, k0, len, m, sm.row, rec, nrec);
+    // the steps pass in groups of G steps: a group in which no lane of the warp jumps runs
+    // straight; the others step by step, the jump paths' code once per control (a copy per
+    // step of a group as well overflowed the instruction cache: paired sweep at lambda dt =
+    // 0.1 5.2 against 3.8 ms, M = 2^20, N_t = 160; one copy for both controls, their values
+    // swapped through it, cost more than it saved: 2.3 against 1.8 ms at 0.01)
+    constexpr int G = SV > 1 ? SV : 2;
+    int rr = 0;
+#pragma unroll 1
+    for (int ii = 0; ii < len; ii += G) {
+      if (((cb.any >> ii) & ((1u << G) - 1u)) == 0u && ii + G <= len) {
+#pragma unroll
+        for (int q = 0; q < G; ++q) {
+          const int k = k0 + ii + q;
+          R z[D], xk[D];
+          get_normals<R, D>(sm.row, ii + q, z);
+          load_row<R, D>(xd + (size_t)(k + 1) * D, xk);
+#pragma unroll
+          for (int h = 0; h < NC; ++h) {
+            if (MODE == FWD_STORE)
+#pragma unroll
+              for (int c = 0; c < D; ++c) buf[h][q % SV][c] = x[h][c];
+            if (MODE == FWD_STORE && q % SV == SV - 1 && active)
+              store_group<R, D>(h ? p2.traj : traj, k / SV, mloc, lm, buf[h]);
+            R uk[DU], f[D];
+#pragma unroll
+            for (int l = 0; l < DU; ++l) uk[l] = __ldg((h ? p2.u : u) + (size_t)k * DU + l);
+            drift(kh, x[h], uk, f);
+            plain_update(kh, f, z, x[h]);
+            cost[h].add(cost_term_row(kh, x[h], xk));
+          }
+        }
+        continue;
+      }
+#pragma unroll 1
+      for (int i = ii; i < min(ii + G, len); ++i) {
+        const int k = k0 + i;
+        R z[D], xk[D];
+        get_normals<R, D>(sm.row, i, z);
+        load_row<R, D>(xd + (size_t)(k + 1) * D, xk);
+        if (MODE == FWD_STORE) {
+#pragma unroll
+          for (int h = 0; h < NC; ++h) {
+#pragma unroll
+            for (int q = 0; q < SV; ++q)
+#pragma unroll
+              for (int c = 0; c < D; ++c) buf[h][q][c] = k % SV == q ? x[h][c] : buf[h][q][c];
+            if (k % SV == SV - 1 && active) store_group<R, D>(h ? p2.traj : traj, k / SV, mloc, lm, buf[h]);
+          }
+        }
+        const bool jumped = (cb.jump >> i) & 1u;
+        const int nr = cb.records(i);
+#pragma unroll
+        for (int h = 0; h < NC; ++h) {
+          R uk[DU];
+#pragma unroll
+          for (int l = 0; l < DU; ++l) uk[l] = __ldg((h ? p2.u : u) + (size_t)k * DU + l);
+          chunk_step(kp, kh, k, m, jumped, nr, rec + rr * FwdChunk<R, D>::W, z, uk, x[h], lw[h]);
+          cost[h].add(cost_term_row(kh, x[h], xk));
+        }
+        rr += nr;
+      }
+    }
+    if constexpr (MODE == FWD_STORE) {
+      fw |= cb.jump << (k0 & 31);
+      if (((k0 + L) & 31) == 0 || k0 + L >= Nt) {
+        if (active) flags[(size_t)(k0 >> 5) * mloc + lm] = fw;
+        fw = 0;
+      }
+    }
+  }
+  if constexpr (MODE == FWD_STORE) {
+    if (active) {   // the last group: X_Nt at its position, zeros after it
+      const int j = Nt % SV;
+#pragma unroll
+      for (int h = 0; h < NC; ++h) {
+#pragma unroll
+        for (int q = 0; q < SV; ++q)
+#pragma unroll
+          for (int c = 0; c < D; ++c) buf[h][q][c] = q == j ? x[h][c] : (q < j ? buf[h][q][c] : R(0));
+        store_group<R, D>(h ? p2.traj : traj, Nt / SV, mloc, lm, buf[h]);
+      }
+      jcnt[lm] = lw[0].r;   // the same count and closing step for the second control
+      jcnt[mloc + lm] = min(lw[0].kovf, Nt);
+    }
+  }
+  if (MODE == FWD_CKPT && active) {
+    const int nseg = (Nt + kp.S - 1) / kp.S;
+#pragma unroll
+    for (int h = 0; h < NC; ++h)
+#pragma unroll
+      for (int c = 0; c < D; ++c) (h ? p2.ckpt : ckpt)[((size_t)nseg * D + c) * mloc + lm] = x[h][c];
+  }
+#pragma unroll
+  for (int h = 0; h < NC; ++h) {
+    Pair<R> v = cost[h].pair();
+    if (!active) v = {R(0), R(0)};
+    if (h == 0 && pcost && active) pcost[lm] = M::add(v.s, v.e);
+    const double sum = block_sum_to_double(v, red);
+    if (tid == 0) (h ? p2.partC : partC)[bid] = sum;
+  }
+}
+
 // The cost partials of a spread sweep: block b of TPB threads takes the pairs of paths
 // b TPB .. b TPB + TPB - 1 (the zero pair past mloc, as an idle thread of the sweep has) and
 // sums them with block_sum_to_double, so partC[b] is the one-path-per-thread sweep's.
@@ -1181,7 +1605,7 @@ __global__ void __launch_bounds__(TPB) spread_combine_kernel(const Pair<R> *__re
   }
 }
 
-template <typename R, int D, int DU, int MODE, bool PAIR = false, bool PRE = false>
+template <typename R, int D, int DU, int MODE, bool PAIR = false, bool PRE = false, bool CHUNK = false>
 __global__ void __launch_bounds__(TPB)
 fwd_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u,
            const R *__restrict__ xd, double *__restrict__ partC, R *__restrict__ traj,
@@ -1204,6 +1628,10 @@ fwd_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u
                                           second ? p2.traj : traj, second ? nullptr : flags,
                                           second ? p2.ckpt : ckpt, nullptr, second ? p2.jl : jl,
                                           second ? nullptr : jcnt, mloc, PairOut<R, D>{}, pd1, red);
+  } else if constexpr (CHUNK) {
+    __shared__ FwdChunkSmem<R, D, PAIR> sm;
+    fwd_chunk_body<R, D, DU, MODE, PAIR, true, PAIR ? 1 : 2>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt,
+                                               mloc, p2, sm, red);
   } else {
     fwd_body<R, D, DU, MODE, PAIR, PRE, RK>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt, mloc,
                                             p2, pd, red);
@@ -1488,6 +1916,9 @@ __host__ __device__ constexpr int seg_log_cap() {
 }
 
 
+// Slot records per path of a replay chunk (d <= 2).
+constexpr int RCREC = 2;
+
 // The parameter-gradient variant of the recompute adjoint keeps each step's normals
 // from the forward replay (instead of drawing them again) when the doubled segment
 // buffer still leaves room for two or more blocks per SM.
@@ -1497,13 +1928,25 @@ __host__ __device__ constexpr bool recompute_zbuf() {
                           (size_t)seg_log_cap<D>() * (2 + D) * TPB * sizeof(R) <= 100 * 1024;
 }
 
+// State i of a segment: in the layout of put_normals (VEC) or one row per component.
+template <typename R, int D, bool VEC>
+__device__ __forceinline__ void seg_state(const R *sbuf, int i, R (&x)[D]) {
+  const R(*const row)[TPB] = reinterpret_cast<const R(*)[TPB]>(sbuf);
+  if constexpr (VEC) {
+    get_normals<R, D>(row, i, x);
+  } else {
+#pragma unroll
+    for (int c = 0; c < D; ++c) x[c] = row[i * D + c][threadIdx.x];
+  }
+}
+
 // Recompute adjoint.  Per segment of S steps (a multiple of 8): replay the forward from
 // the checkpoint into shared memory (states, a short jump log, and for the parameter
 // gradients the main-stream normals), then sweep the segment backwards in chunks of 8
 // steps, each in the fast form of the stored adjoint when no lane of the warp meets a
 // jump step the segment's log does not hold.  Same step arithmetic and the same gradient
 // tree as the stored adjoint (with 8-step rows, half the shared memory): the same bits.
-template <typename R, int D, int DU, bool THETA>
+template <typename R, int D, int DU, bool THETA, bool RCH>
 __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, const R *__restrict__ u,
                                                    const R *__restrict__ xd, const R *__restrict__ ckpt,
                                                    double *__restrict__ partG, double *__restrict__ partT,
@@ -1524,6 +1967,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
   constexpr int NR = 8;
   GradRows<R, DU, NR> rows;
   rows.init(sy + (size_t)JS * D * TPB);
+  R(*const srec)[TPB] = reinterpret_cast<R(*)[TPB]>(sy + (size_t)JS * D * TPB + grad_rows_bytes<R, DU, 8>() / sizeof(R));
   __shared__ Pair<R> red1[TPB / 32];
   const int64_t npart = kp.npart;
   const int64_t lm = (int64_t)blockIdx.x * TPB + threadIdx.x;
@@ -1555,13 +1999,43 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
       lw.L = sl;
       lw.idx = tid;
     }
+    if constexpr (RCH) {
+      // chunks of the replay: the step's normals wait where its state will lie
 #pragma unroll 1
-    for (int i = 0; i < len; ++i) {
+      for (int c0 = 0; c0 < len; c0 += kp.chunk) {
+        const int clen = min(kp.chunk, len - c0);
+        R(*const col)[TPB] = reinterpret_cast<R(*)[TPB]>(sbuf + (size_t)c0 * D * TPB);
+        const ChunkBits cb = chunk_draws<R, D, DU, 1, true>(kp, k0 + c0, clen, m, col, srec, RCREC);
+        jm |= (uint64_t)cb.jump << c0;
+        int rr = 0;
+#pragma unroll 1
+        for (int i = 0; i < clen; ++i) {
+          const int k = k0 + c0 + i;
+          R z[D], uk[DU];
+          get_normals<R, D>(col, i, z);
+          put_normals<R, D>(col, i, x);
 #pragma unroll
-      for (int c = 0; c < D; ++c) sbuf[(i * D + c) * TPB + tid] = x[c];
-      if (forward_step<R, D, DU, LWR, ZBUF, !THETA>(kp, k0 + i, m, u, x, lw, zbuf + (size_t)i * D * TPB + tid,
-                                                    TPB))
-        jm |= 1ull << i;
+          for (int l = 0; l < DU; ++l) uk[l] = __ldg(u + (size_t)k * DU + l);
+          if ((cb.any >> i) & 1u) {
+            const int nrec = cb.records(i);
+            chunk_step(kp, kp, k, m, (cb.jump >> i) & 1u, nrec, srec + rr * FwdChunk<R, D>::W, z, uk, x, lw);
+            rr += nrec;
+          } else {
+            R f[D];
+            drift(kp, x, uk, f);
+            plain_update(kp, f, z, x);
+          }
+        }
+      }
+    } else {
+#pragma unroll 1
+      for (int i = 0; i < len; ++i) {
+  #pragma unroll
+        for (int c = 0; c < D; ++c) sbuf[(i * D + c) * TPB + tid] = x[c];
+        if (forward_step<R, D, DU, LWR, ZBUF, !THETA>(kp, k0 + i, m, u, x, lw, zbuf + (size_t)i * D * TPB + tid,
+                                                      TPB))
+          jm |= 1ull << i;
+      }
     }
     LogReader2<R, D> lr;
     int kovf = 0;
@@ -1590,8 +2064,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
         for (int j = CH - 1; j >= 0; --j) {
           const int i = i0 + j;
           R g[DU], xk[D], xdk[D];
-#pragma unroll
-          for (int c = 0; c < D; ++c) xk[c] = sbuf[(i * D + c) * TPB + tid];
+          seg_state<R, D, RCH>(sbuf, i, xk);
           load_row<R, D>(xdc + j * D, xdk);
           backward_logged(kp, xk, mu, g, lr, (jwm >> j) & 1u, (jm >> i) & 1u);
           cost_gradient(kp, xk, xdk, mu);
@@ -1607,8 +2080,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
           for (int l = 0; l < DU; ++l) g[l] = R(0);
           if (i < len) {
             R xk[D];
-#pragma unroll
-            for (int c = 0; c < D; ++c) xk[c] = sbuf[(i * D + c) * TPB + tid];
+            seg_state<R, D, RCH>(sbuf, i, xk);
             const bool jumped = (jm >> i) & 1u;
             if constexpr (THETA) {
               backward_step<R, D, DU, true, LogReader<R, D>, ZBUF>(kp, kp, k, m, jumped, xk, u, xd, mu, g, th, lr0,
@@ -1644,8 +2116,8 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
 //   replay  the states from the checkpoint, a one-jump step from its record;
 //   back    the adjoint; a one-jump step's post-jump state is formed again from X_k and the
 //           record (the replay's operations: the same bits).
-// Steps with several jumps and one-jump steps beyond THETA_RECS records are regenerated by
-// jump_backward.  At lambda dt = 0.01 a lane has more than two one-jump steps in 16 with
+// Steps with several jumps are regenerated by jump_backward, one-jump steps beyond the
+// records draw their slot again.  At lambda dt = 0.01 a lane has more than two one-jump steps in 16 with
 // probability 6e-4.  Bound by instruction issue.  Before, the replay drew a jump step's slot
 // in divergent code per step and the backward regenerated every jump step through
 // jump_backward: 39.1 -> 13.8 ms per launch at M = 2^20, N_t = 1024, lambda dt = 0.0098 (27%
@@ -1695,8 +2167,7 @@ __device__ __forceinline__ void theta_substep(const KParams<R, D, DU> &kp, const
 template <typename R, int D, int DU>
 __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, const R *__restrict__ u,
                                                const R *__restrict__ xd, const R *__restrict__ ckpt,
-                                               double *__restrict__ partG, double *__restrict__ partT,
-                                               int64_t mloc) {
+                                               double *__restrict__ partG, double *__restrict__ partT, int64_t mloc) {
   using M = Ar<R>;
   constexpr int CH = 8, NR = 8;
   extern __shared__ __align__(16) unsigned char dsm[];
@@ -1731,8 +2202,8 @@ __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, cons
     R x[D];
 #pragma unroll
     for (int c = 0; c < D; ++c) x[c] = __ldg(ckpt + ((size_t)seg * D + c) * mloc + lmc);
-    // bit i: step k0 + i had jumps (jm); exactly one (om) (S <= 64)
-    uint64_t jm = 0, om = 0;
+    // bit i: step k0 + i had jumps (jm); exactly one (om1) (S <= 64)
+    uint64_t jm = 0, om1 = 0;
 #pragma unroll 1
     for (int i = 0; i < len; ++i) {
       R z[D];
@@ -1741,10 +2212,10 @@ __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, cons
       for (int c = 0; c < D; ++c) zbuf[(i * D + c) * TPB + tid] = z[c];
       if (has_jump(kp, w0)) {
         jm |= 1ull << i;
-        if (one_jump(kp, w0)) om |= 1ull << i;
+        if (one_jump(kp, w0)) om1 |= 1ull << i;
       }
     }
-    uint64_t rm = 0;   // steps with a record, in record order
+    uint64_t rm = 0, om = om1;   // rm: steps with a record, in record order
 #pragma unroll 1
     for (int r = 0; r < ThetaRecs<R, D>::N; ++r) {
       if (om == 0) continue;
@@ -1775,13 +2246,17 @@ __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, cons
         R f[D];
         drift(kp, x, uk, f);
         plain_update(kp, f, z, x);
-      } else if ((rm >> i) & 1u) {
+      } else if ((om1 >> i) & 1u) {
         R xih[D], z1[D];
-        const R t1 = rec.load(rr++, xih, z1);
+        R t1;
+        if ((rm >> i) & 1u)
+          t1 = rec.load(rr++, xih, z1);
+        else
+          t1 = slot0_draws<true>(kp, k, m, xih, z1);
         euler_substep(kp, M::mul(kp.dt, t1), z, uk, x);
         apply_jump(kp, x, xih);
         euler_substep(kp, M::mul(kp.dt, M::sub(R(1), t1)), z1, uk, x);
-      } else {   // several jumps, or no record left: the general routine, on copies
+      } else {   // several jumps: the general routine, on copies
         JumpStep<R, D> js;
         R xl[D], ul[DU];
 #pragma unroll
@@ -1814,9 +2289,13 @@ __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, cons
           }
           if (!((jm >> i) & 1u)) {
             theta_substep(kp, xk, z, kp.dt, kp.sqdt, mu, g, th);
-          } else if ((rm >> i) & 1u) {
+          } else if ((om1 >> i) & 1u) {
             R xih[D], z1[D], y[D], uk[DU];
-            const R t1 = rec.load(--rr, xih, z1);
+            R t1;
+            if ((rm >> i) & 1u)
+              t1 = rec.load(--rr, xih, z1);
+            else
+              t1 = slot0_draws<true>(kp, k, m, xih, z1);
 #pragma unroll
             for (int l = 0; l < DU; ++l) uk[l] = __ldg(u + (size_t)k * DU + l);
             const R de0 = M::mul(kp.dt, t1), de1 = M::mul(kp.dt, M::sub(R(1), t1));
@@ -1868,26 +2347,31 @@ __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, cons
   finish_theta<R, D, DU, true>(kp, th, active, partT, red1, blockIdx.x);
 }
 
-template <typename R, int D, int DU, bool THETA>
+// CHUNK: the replay in chunks (u-gradient, d <= 2), or the kept jump draws (parameter
+// gradients); the host's rule (op_adj).
+template <typename R, int D, int DU, bool THETA, bool CHUNK = false>
 __global__ void __launch_bounds__(TPB)
 adj_recompute_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u,
                      const R *__restrict__ xd, const R *__restrict__ ckpt,
                      double *__restrict__ partG, double *__restrict__ partT, int64_t mloc) {
-  if constexpr (THETA && recompute_zbuf<R, D, THETA>())
+  if constexpr (THETA && CHUNK)
     adj_theta_body<R, D, DU>(kp, u, xd, ckpt, partG, partT, mloc);
   else
-    adj_recompute_body<R, D, DU, THETA>(kp, u, xd, ckpt, partG, partT, mloc);
+    adj_recompute_body<R, D, DU, THETA, CHUNK>(kp, u, xd, ckpt, partG, partT, mloc);
 }
 
 // The parameter-gradient form for FP32 d <= 2 with at least 5 blocks per SM: the default
 // allocation took 80 registers and spilled; 94 registers without spills run 20.4 -> 17.7
 // ms per launch at M = 2^20, N_t = 1024 (the u-gradient form keeps its own allocation).
-template <typename R, int D, int DU>
+template <typename R, int D, int DU, bool CHUNK>
 __global__ void __launch_bounds__(TPB, 5)
 adj_recompute_theta5_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u,
                             const R *__restrict__ xd, const R *__restrict__ ckpt,
                             double *__restrict__ partG, double *__restrict__ partT, int64_t mloc) {
-  adj_theta_body<R, D, DU>(kp, u, xd, ckpt, partG, partT, mloc);
+  if constexpr (CHUNK)
+    adj_theta_body<R, D, DU>(kp, u, xd, ckpt, partG, partT, mloc);
+  else
+    adj_recompute_body<R, D, DU, true, false>(kp, u, xd, ckpt, partG, partT, mloc);
 }
 
 template <typename R, int D>
@@ -1895,14 +2379,28 @@ constexpr bool theta5() {
   return sizeof(R) == 4 && D <= 2;
 }
 
-// The parameter-gradient recompute kernel an instantiation launches.
+// The recompute kernel of a launch.
 template <typename R, int D, int DU>
-const void *theta_recompute_fn() {
-  if constexpr (theta5<R, D>())
-    return (const void *)adj_recompute_theta5_kernel<R, D, DU>;
-  else
-    return (const void *)adj_recompute_kernel<R, D, DU, true>;
+auto recompute_form(bool theta, bool chunk) {
+  auto k = &adj_recompute_kernel<R, D, DU, false>;
+  if (theta) {
+    if constexpr (theta5<R, D>())
+      k = chunk ? &adj_recompute_theta5_kernel<R, D, DU, true> : &adj_recompute_theta5_kernel<R, D, DU, false>;
+    else if constexpr (recompute_zbuf<R, D, true>())
+      k = chunk ? &adj_recompute_kernel<R, D, DU, true, true> : &adj_recompute_kernel<R, D, DU, true>;
+    else
+      k = &adj_recompute_kernel<R, D, DU, true>;
+  } else if constexpr (fwd_chunked<D>()) {
+    if (chunk) k = &adj_recompute_kernel<R, D, DU, false, true>;
+  }
+  return k;
 }
+
+// Parameter gradients: the jump draws are kept up to this jump rate per step; beyond it a
+// segment's jumps outgrow the records and most steps have several (M = 2^19, N_t = 160, d = 2
+// FP32, regenerated -> kept: 0.80 -> 0.86 ms without jumps, 1.36 -> 0.94 at 0.002, 3.29 ->
+// 1.16 at 0.01, 7.82 -> 4.16 at 0.05, 10.9 -> 9.8 at 0.1, 16.0 -> 20.0 at 0.2).
+constexpr double THETA_KEEP_RATE = 0.12;
 
 // ---------------------------------------------------------------------------
 // Host-side launch ops for one (precision, D, DU)
@@ -1973,6 +2471,8 @@ void make_kparams(const jd_problem *p, int64_t m_begin, int64_t mloc, KParams<R,
   kp.jump_law = (int)q.jump_law;
   kp.jumps_on = q.jump_law != JD_JUMP_NONE && q.lambda > 0.0;
   kp.has_dA = !p->dA.empty();
+  kp.chunk = 4;
+  if constexpr (fwd_chunked<D>()) kp.chunk = fwd_chunk_len(q.lambda * dt, FwdChunk<R, D>::CH);
   kp.S = p->S;   // checkpoint spacing of the recompute plan (a power of two, 16 .. 64)
   kp.nblk = (int)ceil_div(mloc, TPB);
   kp.m_begin = q.m_offset + m_begin;   // global path index (a shard starts at m_offset)
@@ -2001,6 +2501,16 @@ unsigned long long draws_key(const KParams<R, D, DU> &kp, int64_t mloc) {
   mix((unsigned long long)kp.jumps_on);
   for (int n = 0; n < NMAX; ++n) mix(kp.thr[n]);
   return h | 1ull;
+}
+
+// The sweep's kernel: in chunks or step by step.
+template <typename R, int D, int DU, int MODE, bool PAIR = false>
+auto fwd_form(bool chunk) {
+  auto k = &fwd_kernel<R, D, DU, MODE, PAIR>;
+  if constexpr (fwd_chunked<D>()) {
+    if (chunk) k = &fwd_kernel<R, D, DU, MODE, PAIR, false, true>;
+  }
+  return k;
 }
 
 template <typename R, int D, int DU>
@@ -2059,32 +2569,35 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
       return cudaGetLastError();
     }
   }
+  const bool chunk = fwd_chunks<R, D>(p->desc.lambda * p->desc.T / (double)p->desc.Nt, mode == FWD_STORE);
   switch (mode) {
     case FWD_COST:
-      fwd_kernel<R, D, DU, FWD_COST><<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr, nullptr, pc,
-                                                          jl, nullptr, mloc, p2);
+      fwd_form<R, D, DU, FWD_COST>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr, nullptr, pc, jl,
+                                                               nullptr, mloc, p2, PreDraws<R, D>{});
       break;
     case FWD_STORE:
-      fwd_kernel<R, D, DU, FWD_STORE><<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, static_cast<R *>(b.traj),
-                                                           b.flags, nullptr, pc, jl, b.jcnt, mloc, p2);
+      fwd_form<R, D, DU, FWD_STORE>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, static_cast<R *>(b.traj), b.flags,
+                                                                nullptr, pc, jl, b.jcnt, mloc, p2, PreDraws<R, D>{});
       break;
     case FWD_STORE | FWD_PAIR:
     case FWD_CKPT | FWD_PAIR:
       if constexpr (PAIR_SWEEPS<D>) {   // the host asks for pairs only where they are built
         if (mode & FWD_STORE)
-          fwd_kernel<R, D, DU, FWD_STORE, true><<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, static_cast<R *>(b.traj),
-                                                                     b.flags, nullptr, nullptr, jl, b.jcnt, mloc, p2);
+          fwd_form<R, D, DU, FWD_STORE, true>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, static_cast<R *>(b.traj),
+                                                                          b.flags, nullptr, nullptr, jl, b.jcnt, mloc,
+                                                                          p2, PreDraws<R, D>{});
         else
-          fwd_kernel<R, D, DU, FWD_CKPT, true><<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr,
-                                                                    static_cast<R *>(b.ckpt), nullptr, jl, nullptr,
-                                                                    mloc, p2);
+          fwd_form<R, D, DU, FWD_CKPT, true>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr,
+                                                                         static_cast<R *>(b.ckpt), nullptr, jl,
+                                                                         nullptr, mloc, p2, PreDraws<R, D>{});
       } else {
         return cudaErrorNotSupported;
       }
       break;
     default:
-      fwd_kernel<R, D, DU, FWD_CKPT><<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr,
-                                                          static_cast<R *>(b.ckpt), pc, jl, nullptr, mloc, p2);
+      fwd_form<R, D, DU, FWD_CKPT>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr,
+                                                               static_cast<R *>(b.ckpt), pc, jl, nullptr, mloc, p2,
+                                                               PreDraws<R, D>{});
       break;
   }
   count_launch();
@@ -2092,11 +2605,20 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
 }
 
 // Shared memory of the recompute adjoint for segments of S steps.
+// (chunk: the form with records, recompute_form's).
+template <typename R, int D, int DU>
+size_t recompute_smem_form(bool theta, bool chunk, int S) {
+  const bool zbuf = theta && recompute_zbuf<R, D, true>();
+  size_t n = (size_t)S * D * TPB * sizeof(R) * (zbuf ? 2 : 1) + grad_rows_bytes<R, DU, 8>();
+  if (!theta) n += (size_t)seg_log_cap<D>() * (2 + D) * TPB * sizeof(R);
+  if (zbuf && chunk) n += theta_rec_bytes<R, D>();
+  if (!theta && chunk && fwd_chunked<D>()) n += (size_t)RCREC * FwdChunk<R, D>::W * TPB * sizeof(R);
+  return n;
+}
+// The larger of the two forms (the plan's choice of S).
 template <typename R, int D, int DU>
 size_t recompute_smem(bool theta, int S) {
-  const bool zbuf = theta && recompute_zbuf<R, D, true>();
-  return (size_t)S * D * TPB * sizeof(R) * (zbuf ? 2 : 1) + (zbuf ? theta_rec_bytes<R, D>() : 0) +
-         (theta ? 0 : (size_t)seg_log_cap<D>() * (2 + D) * TPB * sizeof(R)) + grad_rows_bytes<R, DU, 8>();
+  return recompute_smem_form<R, D, DU>(theta, true, S);
 }
 
 // The dynamic shared-memory limit of a kernel is an attribute of the function on the
@@ -2150,23 +2672,13 @@ cudaError_t op_adj(const jd_problem *p, int variant, bool theta, int64_t m_begin
                                                                    b.partT, nullptr, mloc);
     }
   } else {
-    const size_t smem = recompute_smem<R, D, DU>(theta, kp.S);
     const R *ck = static_cast<const R *>(b.ckpt);
-    if (theta) {
-      if constexpr (theta5<R, D>()) {
-        err = ensure_dyn_smem((const void *)adj_recompute_theta5_kernel<R, D, DU>, smem);
-        if (err == cudaSuccess)
-          adj_recompute_theta5_kernel<R, D, DU><<<grid, TPB, smem, s>>>(kp, u, xd, ck, b.partG, b.partT, mloc);
-      } else {
-        err = ensure_dyn_smem((const void *)adj_recompute_kernel<R, D, DU, true>, smem);
-        if (err == cudaSuccess)
-          adj_recompute_kernel<R, D, DU, true><<<grid, TPB, smem, s>>>(kp, u, xd, ck, b.partG, b.partT, mloc);
-      }
-    } else {
-      err = ensure_dyn_smem((const void *)adj_recompute_kernel<R, D, DU, false>, smem);
-      if (err == cudaSuccess)
-        adj_recompute_kernel<R, D, DU, false><<<grid, TPB, smem, s>>>(kp, u, xd, ck, b.partG, b.partT, mloc);
-    }
+    const double lamdt = p->desc.lambda * p->desc.T / (double)p->desc.Nt;
+    const bool chunk = theta ? lamdt <= THETA_KEEP_RATE : fwd_chunks<R, D>(lamdt, false);
+    const size_t smem = recompute_smem_form<R, D, DU>(theta, chunk, kp.S);
+    const auto k = recompute_form<R, D, DU>(theta, chunk);
+    err = ensure_dyn_smem((const void *)k, smem);
+    if (err == cudaSuccess) k<<<grid, TPB, smem, s>>>(kp, u, xd, ck, b.partG, b.partT, mloc);
   }
   count_launch();
   if (err != cudaSuccess) return err;
@@ -2205,13 +2717,17 @@ __device__ __forceinline__ int sweep_item(const int *first, int n) {
   return i;
 }
 
+// 80 registers, the pair 128, since the coefficients are read through the table; bounded for
+// more resident blocks it was slower.  12 small requests of 3 iterations: 7.57 ms step by
+// step, 6.78 in chunks.
 template <typename R, int D, int DU, bool PAIR>
 __global__ void __launch_bounds__(TPB) fwd_batch_kernel(const __grid_constant__ SweepBatch<R, D, DU> t) {
   __shared__ Pair<R> red[TPB / 32];
   const int i = sweep_item(t.first, t.n);
   const SweepItem<R, D, DU> &f = t.it[i];
-  fwd_body<R, D, DU, FWD_STORE, PAIR, false>(f.kp, blockIdx.x - t.first[i], f.u, f.xd, f.partC, f.traj, f.flags,
-                                             nullptr, nullptr, f.jl, f.jcnt, f.mloc, f.p2, PreDraws<R, D>{}, red);
+  __shared__ FwdChunkSmem<R, D, PAIR> sm;
+  fwd_chunk_body<R, D, DU, FWD_STORE, PAIR, false, 1>(f.kp, blockIdx.x - t.first[i], f.u, f.xd, f.partC, f.traj, f.flags,
+                                                   nullptr, nullptr, f.jl, f.jcnt, f.mloc, f.p2, sm, red);
 }
 
 template <typename R, int D, int DU>
@@ -2307,19 +2823,23 @@ template <typename R, int D, int DU>
 size_t op_stack_bytes() {
   size_t need = 2 * sizeof(JumpStep<R, D>) + 2048;
   const void *ks[] = {
-      (const void *)fwd_kernel<R, D, DU, FWD_COST>, (const void *)fwd_kernel<R, D, DU, FWD_STORE>,
-      (const void *)fwd_kernel<R, D, DU, FWD_CKPT>, (const void *)adj_stored_kernel<R, D, DU, false>,
-      (const void *)adj_stored_kernel<R, D, DU, false, true>,
-      (const void *)adj_stored_kernel<R, D, DU, true>, (const void *)adj_recompute_kernel<R, D, DU, false>,
-      theta_recompute_fn<R, D, DU>()};
+      (const void *)fwd_form<R, D, DU, FWD_COST>(false), (const void *)fwd_form<R, D, DU, FWD_STORE>(false),
+      (const void *)fwd_form<R, D, DU, FWD_CKPT>(false), (const void *)fwd_form<R, D, DU, FWD_COST>(true),
+      (const void *)fwd_form<R, D, DU, FWD_STORE>(true), (const void *)fwd_form<R, D, DU, FWD_CKPT>(true),
+      (const void *)adj_stored_kernel<R, D, DU, false>, (const void *)adj_stored_kernel<R, D, DU, false, true>,
+      (const void *)adj_stored_kernel<R, D, DU, true>, (const void *)recompute_form<R, D, DU>(false, false),
+      (const void *)recompute_form<R, D, DU>(false, true), (const void *)recompute_form<R, D, DU>(true, false),
+      (const void *)recompute_form<R, D, DU>(true, true)};
   for (const void *k : ks) {
     cudaFuncAttributes a;
     if (cudaFuncGetAttributes(&a, k) == cudaSuccess && a.localSizeBytes + 1024 > need)
       need = a.localSizeBytes + 1024;
   }
   if constexpr (PAIR_SWEEPS<D>) {
-    for (const void *k : {(const void *)fwd_kernel<R, D, DU, FWD_STORE, true>,
-                          (const void *)fwd_kernel<R, D, DU, FWD_CKPT, true>}) {
+    for (const void *k : {(const void *)fwd_form<R, D, DU, FWD_STORE, true>(false),
+                          (const void *)fwd_form<R, D, DU, FWD_CKPT, true>(false),
+                          (const void *)fwd_form<R, D, DU, FWD_STORE, true>(true),
+                          (const void *)fwd_form<R, D, DU, FWD_CKPT, true>(true)}) {
       cudaFuncAttributes a;
       if (cudaFuncGetAttributes(&a, k) == cudaSuccess && a.localSizeBytes + 1024 > need)
         need = a.localSizeBytes + 1024;

@@ -111,6 +111,7 @@ static void noalloc_kparams(const jd_problem_desc &q, KParams<R, D, DU> &kp) {
   kp.jumps_on = q.jump_law != JD_JUMP_NONE && q.lambda > 0.0;
   kp.has_dA = 0;
   kp.S = seg_len<D>();
+  kp.chunk = fwd_chunk_len(q.lambda * dt, FwdChunk<R, D>::CH);
   kp.nblk = (int)ceil_div(q.M, TPB);
   kp.m_begin = q.m_offset;   // global index of the first path
   kp.npart = kp.nblk * (int64_t)(TPB / 32);
@@ -140,8 +141,9 @@ static jd_status noalloc_run(const jd_problem_desc &q, unsigned char *scratch, c
   KParams<R, D, 1> kp;
   noalloc_kparams<R, D, 1>(q, kp);
   const JLog<R, D> nolog{nullptr, nullptr, M, 0};
-  fwd_kernel<R, D, 1, FWD_COST><<<(unsigned)nblk, TPB, 0, s>>>(kp, uk, xdk, partC, nullptr, nullptr, nullptr,
-                                                               nullptr, nolog, nullptr, M, PairOut<R, D>{});
+  const auto k = fwd_form<R, D, 1, FWD_COST>(fwd_chunks<R, D>(q.lambda * (q.T / (double)Nt), false));
+  k<<<(unsigned)nblk, TPB, 0, s>>>(kp, uk, xdk, partC, nullptr, nullptr, nullptr, nullptr, nolog, nullptr, M,
+                                   PairOut<R, D>{}, PreDraws<R, D>{});
   noalloc_finalize_kernel<<<1, 256, 0, s>>>(partC, nblk, u, Nt, 0.5 * q.nu * (q.T / Nt), 1.0 / (double)M, J);
   count_launch(3);
   return cudaGetLastError() == cudaSuccess ? JD_OK : JD_ERR_CUDA;
@@ -183,14 +185,16 @@ extern "C" jd_status jd_cost_noalloc(const jd_problem_desc *desc, const double *
     if (!g_noalloc_ptr[dev]) {
       void *ptr = nullptr;
       if (cudaGetSymbolAddress(&ptr, g_noalloc_scratch) != cudaSuccess || !ptr) return JD_ERR_CUDA;
-      const void *ks[4] = {(const void *)fwd_kernel<float, 1, 1, FWD_COST>,
-                           (const void *)fwd_kernel<float, 2, 1, FWD_COST>,
-                           (const void *)fwd_kernel<double, 1, 1, FWD_COST>,
-                           (const void *)fwd_kernel<double, 2, 1, FWD_COST>};
-      for (int i = 0; i < 4; ++i) {
-        cudaFuncAttributes a;
-        if (cudaFuncGetAttributes(&a, ks[i]) != cudaSuccess) return JD_ERR_CUDA;
-        g_noalloc_stack[dev][i] = a.localSizeBytes;
+      for (int chunk = 0; chunk < 2; ++chunk) {   // both forms of each cost kernel
+        const void *ks[4] = {(const void *)fwd_form<float, 1, 1, FWD_COST>(chunk),
+                             (const void *)fwd_form<float, 2, 1, FWD_COST>(chunk),
+                             (const void *)fwd_form<double, 1, 1, FWD_COST>(chunk),
+                             (const void *)fwd_form<double, 2, 1, FWD_COST>(chunk)};
+        for (int i = 0; i < 4; ++i) {
+          cudaFuncAttributes a;
+          if (cudaFuncGetAttributes(&a, ks[i]) != cudaSuccess) return JD_ERR_CUDA;
+          if (a.localSizeBytes > g_noalloc_stack[dev][i]) g_noalloc_stack[dev][i] = a.localSizeBytes;
+        }
       }
       g_noalloc_ptr[dev] = static_cast<unsigned char *>(ptr);
     }

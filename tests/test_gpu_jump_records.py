@@ -42,3 +42,41 @@ def test_parameter_gradients_recompute_equals_stored(model, prec, Nt, lamdt):
             out.append(jp.gradient(u, theta=True))
     for a, b in zip(*out):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("model", ["double_well", "lq_scalar", "ks_oscillator", "ks_scalar"])
+@pytest.mark.parametrize("Nt,lamdt", [(1, 0.3), (3, 0.01), (16, 0.01), (35, 0.02), (61, 0.05), (37, 0.9), (33, 0.0)])
+def test_chunked_sweeps_equal_the_pre_drawn_ones(model, prec, Nt, lamdt):
+    """A problem of many paths runs its sweeps in chunks; its shards are small enough for the
+    pre-drawn sweeps, which go step by step.  The path reduction is defined on units, so the
+    shards' unit sums are the whole problem's bit for bit."""
+    p, u = _problem(model, 2 * 16384 + 7001, Nt, lamdt)
+    with JdProblem(p, prec=prec, mode="stored") as jp:
+        whole, cost = jp.gradient_units(u), jp.cost_units(u)
+    with JdProblem(p, prec=prec, mode="recompute") as jp:
+        again = jp.gradient_units(u)
+    parts, pcost = [], []
+    for m0 in range(0, p.M, 16384):
+        q = p.replace(M=min(16384, p.M - m0), m_offset=m0)
+        with JdProblem(q, prec=prec, mode="stored") as jp:
+            parts.append(jp.gradient_units(u))
+            pcost.append(jp.cost_units(u))
+    assert np.array_equal(whole, np.concatenate(parts))
+    assert np.array_equal(again, whole)
+    assert np.array_equal(cost, np.concatenate(pcost))
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("lamdt", [0.003, 0.05, 0.6])
+def test_chunked_pairs_equal_single_trials(prec, lamdt):
+    """Paired trials run both controls in one chunked sweep: the iterates of single trials."""
+    p, u = _problem("double_well", 40001, 45, lamdt)
+    out = []
+    for mode in ("stored", "recompute"):
+        for pairs in (True, False):
+            with JdProblem(p, prec=prec, mode=mode) as jp:
+                v, r, hist = jp.optimize(u0=u, max_iter=3, tol_rel_grad=0.0, pairs=pairs)
+            out.append((v, hist, r["evals"]))
+    for v, hist, evals in out[1:]:
+        assert np.array_equal(v, out[0][0]) and np.array_equal(hist, out[0][1]) and evals == out[0][2]
