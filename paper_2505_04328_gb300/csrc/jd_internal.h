@@ -137,11 +137,18 @@ inline int ring_lanes(int N) {
 }
 constexpr int RING_MAX = 2048;   // 8 blocks of 256 lanes: the largest portable cluster
 
-// Draw pre-pass: a problem with d <= 2 whose paths fill at most 2 blocks per SM of a
-// GB300 (its sweeps are latency-bound: each thread's steps are a chain of dependent
-// operations, and the Philox and Box-Muller of every step sit on that chain) takes its
-// main-stream draws in one parallel kernel first, when their buffers stay small.
-constexpr int64_t PRE_MAX_PATHS = 152 * 2 * 128;
+// Draw pre-pass: a problem with d <= 2 of few paths (its sweeps are latency-bound: each
+// thread's steps are a chain of dependent operations, and the Philox and Box-Muller of every
+// step sit on that chain) takes its main-stream draws in one parallel kernel first, when
+// their buffers stay small.  Its sweeps then run few lanes per warp (SPREAD_LANES), which
+// costs them instruction issue as the paths grow: the limits are where three projected-
+// gradient iterations take as long with the chunked sweeps (N_t = 200, lambda dt = 0.02,
+// pre-drawn / chunked in us):
+//   FP32 d = 1  M = 4000  805 / 897    8000  903 / 939    16000  1180 / 955   32000  2144 / 1062
+//   FP32 d = 2            817 / 914          946 / 972           1394 / 1009
+//   FP64 d = 1           2246 / 3873        3585 / 3900          6239 / 4002
+//   FP64 d = 2           4106 / 5453        6592 / 5490
+inline int64_t pre_max_paths(int D, size_t es) { return es == 4 ? 152 * 64 : D == 1 ? 152 * 48 : 152 * 32; }
 constexpr size_t PRE_MAX_BYTES = (size_t)128 << 20;
 // pre_z holds the normals, the slot-0 draws and then the paths' cost pairs of the sweeps
 // (2 controls x M pairs of 2 values)
@@ -154,7 +161,7 @@ inline size_t pre_bytes(int Nt, int D, int64_t M, size_t es) {
 }
 inline bool pre_pass(int d, int Nt, int64_t M, size_t es) {
   const int D = d <= 1 ? 1 : 2;
-  return d <= 2 && M <= PRE_MAX_PATHS && pre_bytes(Nt, D, M, es) <= PRE_MAX_BYTES;
+  return d <= 2 && M <= pre_max_paths(D, es) && pre_bytes(Nt, D, M, es) <= PRE_MAX_BYTES;
 }
 
 struct FbBufs {
