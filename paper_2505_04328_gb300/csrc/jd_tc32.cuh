@@ -87,9 +87,10 @@ __device__ __forceinline__ void tc_write_row(unsigned char *hi, unsigned char *l
 }
 
 // Shared state of a tensor-core tile.
+template <bool SPLIT>
 struct TcShared {
-  unsigned char xhi[8192], xlo[8192];   // 128 x 32 BF16 operand tiles (rows = paths)
-  unsigned char ahi[2048], alo[2048];   // 32 x 32 BF16 coefficient tiles
+  unsigned char xhi[8192], xlo[SPLIT ? 8192 : 16];   // 128 x 32 BF16 operand tiles (rows = paths)
+  unsigned char ahi[2048], alo[SPLIT ? 2048 : 16];   // 32 x 32 BF16 coefficient tiles
   unsigned long long mbar;
   uint32_t tmem;
   int stop;     // set when a wait timed out; read by every thread after the issue barrier
@@ -99,7 +100,7 @@ struct TcShared {
 // Write the coefficient tile: row n, column k holds coef(n, k) (A for the forward,
 // A^T for the adjoint).  Threads 0..31 write one row each.
 template <bool SPLIT>
-__device__ __forceinline__ void tc_write_coef(TcShared &sh, const KP32 &kp, bool transpose) {
+__device__ __forceinline__ void tc_write_coef(TcShared<SPLIT> &sh, const KP32 &kp, bool transpose) {
   if (threadIdx.x < 32) {
     float row[32];
     const int n = threadIdx.x;
@@ -109,7 +110,8 @@ __device__ __forceinline__ void tc_write_coef(TcShared &sh, const KP32 &kp, bool
   }
 }
 
-__device__ __forceinline__ void tc_setup(TcShared &sh) {
+template <bool SPLIT>
+__device__ __forceinline__ void tc_setup(TcShared<SPLIT> &sh) {
   if (threadIdx.x < 32) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sh.tmem)),
                  "r"(32));
@@ -124,7 +126,8 @@ __device__ __forceinline__ void tc_setup(TcShared &sh) {
 }
 
 // Bounded wait for mbarrier phase `parity`; true when it completed.
-__device__ __forceinline__ bool tc_wait(TcShared &sh, uint32_t parity) {
+template <bool SPLIT>
+__device__ __forceinline__ bool tc_wait(TcShared<SPLIT> &sh, uint32_t parity) {
   uint32_t done = 0;
   for (int it = 0; it < (1 << 24) && !done; ++it) {
     asm volatile(
@@ -137,7 +140,8 @@ __device__ __forceinline__ bool tc_wait(TcShared &sh, uint32_t parity) {
 
 // Free the tile's tensor memory.  A CTA that stopped after a timed-out wait first waits
 // once more (bounded) for its last product so no MMA is in flight.
-__device__ __forceinline__ void tc_teardown(TcShared &sh) {
+template <bool SPLIT>
+__device__ __forceinline__ void tc_teardown(TcShared<SPLIT> &sh) {
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (sh.stop && threadIdx.x == 0 && sh.issued > 0) (void)tc_wait(sh, (uint32_t)((sh.issued - 1) & 1));
@@ -148,7 +152,7 @@ __device__ __forceinline__ void tc_teardown(TcShared &sh) {
 // Issue the step's product (thread 0) after all rows are written.  Returns false (in
 // every thread, read after the barrier) once the tile has stopped.
 template <bool SPLIT>
-__device__ __forceinline__ bool tc_issue(TcShared &sh) {
+__device__ __forceinline__ bool tc_issue(TcShared<SPLIT> &sh) {
   asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
@@ -173,7 +177,8 @@ __device__ __forceinline__ bool tc_issue(TcShared &sh) {
 
 // Wait for the step's product (bounded) and read this thread's lane: out[n] = row . coef_n.
 // Returns false when the wait timed out (the CTA then stops).
-__device__ __forceinline__ bool tc_collect(TcShared &sh, uint32_t parity, float (&out)[32], int *status) {
+template <bool SPLIT>
+__device__ __forceinline__ bool tc_collect(TcShared<SPLIT> &sh, uint32_t parity, float (&out)[32], int *status) {
   const bool done = tc_wait(sh, parity);
   if (!done) {
     sh.stop = 1;
@@ -329,13 +334,15 @@ __device__ __forceinline__ void regen_jump_times(const KP32 &kp, int k, uint32_t
 // zero, as cc_matvec); every component gets the operations of the one-lane routine in the
 // same order, so the same bits.  A lane alone drew 27 blocks and 48 pairs and did all 32
 // components while its warp (and, with the tensor cores, its CTA at the next step's
-// barrier) waited; here it only hands over X_k and A X_k and takes X_{k+1} and Y_1 back.
+// barrier) waited; here it only hands over X_k and A X_k and takes X_{k+1} back; the
+// component lanes write Y_1 to the path's log when it fits (cap).
 // ws: the warp's 32 x TPB floats of vbuf, free at this point of the step (rows: 0-1 main
 // words, 2-4 slot words, 5 main normals, 6 jump sizes, 7 post-jump normals, 8 Y_1, 9 X,
-// 10 A X_k).  Called by every lane of the warp; returns th in the jump lanes.
-__device__ __forceinline__ float coop_one_jumps(const KP32 &kp, const float *at, float *ws, int k, uint32_t m,
-                                                const float *__restrict__ u, unsigned om, float (&x)[32],
-                                                const float (&f)[32], float (&y1)[32]) {
+// 10 A X_k).  Called by every lane of the warp.
+__device__ __forceinline__ void coop_one_jumps(const KP32 &kp, const float *at, float *ws, int k, uint32_t m,
+                                               const float *__restrict__ u, unsigned om, float (&x)[32],
+                                               const float (&f)[32], const JLog<float, D32> &jl, int64_t lm, int cap,
+                                               int nrec) {
   const int lane = threadIdx.x & 31;
   uint32_t *wu = reinterpret_cast<uint32_t *>(ws);
   auto mword = [&](int w) -> uint32_t & { return wu[(w >> 5) * TPB + (w & 31)]; };
@@ -344,11 +351,11 @@ __device__ __forceinline__ float coop_one_jumps(const KP32 &kp, const float *at,
         *fv = ws + 10 * TPB;
   const uint32_t tag = (1u << 24) | (1u << 16);   // jump slot 0
   const bool sizes_normal = kp.jump_law != JD_JUMP_UNIFORM;
-  float th_out = 0.f;
   while (om) {
     const int j = __ffs(om) - 1;
     om &= om - 1;
     const uint32_t mj = __shfl_sync(0xffffffffu, m, j);
+    const int cj = __shfl_sync(0xffffffffu, cap, j), rj = __shfl_sync(0xffffffffu, nrec, j);
     if (lane < 26) {   // lanes 0..8: main blocks 0..8; lanes 9..25: slot blocks 0..16
       const bool slot = lane >= 9;
       const uint32_t b = slot ? (uint32_t)(lane - 9) : (uint32_t)lane;
@@ -405,6 +412,11 @@ __device__ __forceinline__ float coop_one_jumps(const KP32 &kp, const float *at,
     else
       xc = __fadd_rn(xc, __fmul_rn(kp.jump_scale, __fsub_rn(__fmul_rn(2.f, Ar<float>::u01(sword(1 + c))), 1.f)));
     yv[c] = xc;
+    if (rj + 1 <= cj) {   // the post-jump state to the path's log
+      const int64_t lj = lm - lane + j;
+      if (lane == 0) jl.kt[(int64_t)rj * jl.stride + lj] = V2<float>::rec(16 * k, th);
+      jl.y[((int64_t)rj * D32 + c) * jl.stride + lj] = xc;
+    }
     __syncwarp();
     float acc = 0.f;   // (A Y_1)_c
 #pragma unroll 8
@@ -414,15 +426,125 @@ __device__ __forceinline__ float coop_one_jumps(const KP32 &kp, const float *at,
     __syncwarp();
     if (lane == j) {
 #pragma unroll
-      for (int cc = 0; cc < 32; ++cc) {
-        x[cc] = xv[cc];
-        y1[cc] = yv[cc];
-      }
-      th_out = th;
+      for (int cc = 0; cc < 32; ++cc) x[cc] = xv[cc];
     }
     __syncwarp();   // the scratch is the next jump lane's
   }
-  return th_out;
+}
+
+// Any other jump step of a warp (two or more jumps, or a slot layout of fewer than 16 pairs),
+// by the whole warp: build_jump_step's operations, one component per lane.  The sub-step's
+// drift is B u_k + A y (control first, then k order), the jumps in time order (equal times by
+// slot).  The post-jump states go to the path's log when all fit (cap).  The out-of-line call
+// that did this before kept its caller's registers, so that no more than four CTAs fitted an
+// SM.  ws rows as coop_one_jumps', 10 jump times by slot, 11 in order, 12 slot order.
+__device__ __forceinline__ void coop_jumps(const KP32 &kp, const float *at, float *ws, int k, uint32_t m,
+                                           uint32_t w0, const float *__restrict__ u, unsigned om, float (&x)[32],
+                                           const JLog<float, D32> &jl, int64_t lm, int cap, int nrec) {
+  const int lane = threadIdx.x & 31, L = lane, P = kp.npair, d = kp.d;
+  uint32_t *wu = reinterpret_cast<uint32_t *>(ws);
+  auto mword = [&](int w) -> uint32_t & { return wu[(w >> 5) * TPB + (w & 31)]; };
+  auto sword = [&](int w) -> uint32_t & { return wu[(2 + (w >> 5)) * TPB + (w & 31)]; };
+  float *zm = ws + 5 * TPB, *zs = ws + 6 * TPB, *zp = ws + 7 * TPB, *yv = ws + 8 * TPB, *xv = ws + 9 * TPB,
+        *ts = ws + 10 * TPB, *to = ws + 11 * TPB;
+  int *ord = reinterpret_cast<int *>(ws + 12 * TPB);
+  while (om) {
+    const int j = __ffs((int)om) - 1;
+    om &= om - 1;
+    const uint32_t mj = __shfl_sync(0xffffffffu, m, j), wj = __shfl_sync(0xffffffffu, w0, j);
+    const int cj = __shfl_sync(0xffffffffu, cap, j), rj = __shfl_sync(0xffffffffu, nrec, j);
+    const int64_t lj = lm - lane + j;
+    int n = 0;
+    for (int i = 0; i < NMAX; ++i) n += ((unsigned long long)wj >= kp.thr[i]) ? 1 : 0;
+    const bool log = rj + n <= cj;
+    __syncwarp();
+    if (L < 9 + n) {   // the main stream's blocks and every slot's first block (its time)
+      const uint32_t tag = L < 9 ? (uint32_t)L : ((1u << 24) | ((uint32_t)(L - 8) << 16));
+      const uint4 o = philox10((uint32_t)k, mj, tag, kp.epoch, kp.key0, kp.key1);
+      if (L < 9) {
+        mword(4 * L) = o.x;
+        mword(4 * L + 1) = o.y;
+        mword(4 * L + 2) = o.z;
+        mword(4 * L + 3) = o.w;
+      } else {
+        ts[L - 9] = Ar<float>::u01(o.x);
+      }
+    }
+    if (lane == j) {
+#pragma unroll
+      for (int c = 0; c < 32; ++c) yv[c] = x[c];
+    }
+    __syncwarp();
+    if (L < 16) {
+      float z0, z1;
+      normal_pair<float>(mword(2 * L + 1), mword(2 * L + 2), z0, z1);
+      zm[2 * L] = z0;
+      zm[2 * L + 1] = z1;
+    } else if (L < 16 + n) {
+      const int i = L - 16;
+      const float t = ts[i];
+      int rank = 0;
+      for (int q = 0; q < n; ++q) rank += ts[q] < t || (ts[q] == t && q < i) ? 1 : 0;
+      to[rank] = t;
+      ord[rank] = i;
+    }
+    __syncwarp();
+    float bc = 0.f, y = yv[lane];
+#pragma unroll
+    for (int l = 0; l < DU32; ++l) bc = __fmaf_rn(kp.B[lane * DU32 + l], __ldg(u + (size_t)k * DU32 + l), bc);
+#pragma unroll 1
+    for (int e = 0; e <= n; ++e) {
+      const float prev = e > 0 ? to[e - 1] : 0.f, th = e < n ? to[e] : 1.f;
+      const float de = __fmul_rn(kp.dt, __fsub_rn(th, prev)), z = e == 0 ? zm[lane] : zp[lane];
+      float f = bc;
+#pragma unroll 8
+      for (int kk = 0; kk < 32; ++kk) f = __fmaf_rn(at[kk * 32 + lane], yv[kk], f);
+      y = __fmaf_rn(__fmul_rn(kp.sigma[lane], __fsqrt_rn(de)), z, __fmaf_rn(de, f, y));
+      if (e < n) {   // the slot's sizes (words 1..2P) and next normals (words 1 + 2P..4P)
+        const uint32_t tag = (1u << 24) | ((uint32_t)(ord[e] + 1) << 16);
+        if (L <= P) {
+          const uint4 o = philox10((uint32_t)k, mj, tag | (uint32_t)L, kp.epoch, kp.key0, kp.key1);
+          sword(4 * L) = o.x;
+          sword(4 * L + 1) = o.y;
+          sword(4 * L + 2) = o.z;
+          sword(4 * L + 3) = o.w;
+        }
+        __syncwarp();   // also: every lane has read this sub-step's normals
+        const int q = L & 31;
+        if (L < 2 * P) {
+          const bool post = q >= P;
+          const int p = post ? q - P : q;
+          const uint32_t wa = sword(1 + 2 * q), wb = sword(2 + 2 * q);
+          float a, b;
+          if (!post && kp.jump_law == JD_JUMP_UNIFORM) {
+            a = __fsub_rn(__fmul_rn(2.f, Ar<float>::u01(wa)), 1.f);
+            b = __fsub_rn(__fmul_rn(2.f, Ar<float>::u01(wb)), 1.f);
+          } else {
+            normal_pair<float>(wa, wb, a, b);
+          }
+          float *zo = post ? zp : zs;
+          zo[2 * p] = 2 * p < d ? a : 0.f;
+          zo[2 * p + 1] = 2 * p + 1 < d ? b : 0.f;
+        }
+        __syncwarp();
+        const float xi = lane < d ? zs[lane] : 0.f;
+        y = __fadd_rn(__fmul_rn(kp.jgain[lane], y), __fmul_rn(kp.jscl[lane], xi));
+        if (log) {
+          if (lane == 0) jl.kt[(int64_t)(rj + e) * jl.stride + lj] = V2<float>::rec(16 * k + e, th);
+          jl.y[((int64_t)(rj + e) * D32 + lane) * jl.stride + lj] = y;
+        }
+        if (lane >= d) zp[lane] = 0.f;
+      }
+      __syncwarp();
+      yv[lane] = y;
+      __syncwarp();
+    }
+    __syncwarp();
+    if (lane == j) {
+#pragma unroll
+      for (int c = 0; c < 32; ++c) x[c] = yv[c];
+    }
+  }
 }
 
 // bu[k][c] = sum_l B[c][l] u_k[l] (FP32, multiply-adds in the order l = 0..3 from zero):
@@ -438,6 +560,13 @@ __global__ void bu32_kernel(const KP32 *__restrict__ kpg, const float *__restric
   bu[i] = bc;
 }
 
+// No call in the step loop: with the multi-jump steps out of line the caller kept 128 registers
+// with spills around the call's 32-component copies; without it M = 2^18, N_t = 500 took 12.36
+// -> 11.2 ms with the BF16 product, M = 50,001, N_t = 333, lambda = 2.5 on the CUDA cores 3.00 ->
+// 2.77.  Bound by the latency of dependent instructions, four warps per scheduler.  Tried: two
+// threads per path (components halved, 64 registers, eight warps per scheduler, one more
+// Philox block and every per-thread step twice: 23% more instructions) 14.0 / 3.0 ms, with
+// three CTAs of 256 12.9 / 2.8; five CTAs per SM (96 registers) 11.1 / 3.7.
 template <int TC>
 __global__ void __launch_bounds__(TPB, 4)
 fwd32_kernel(const KP32 *__restrict__ kpg, const float *__restrict__ u, const float *__restrict__ bu,
@@ -446,7 +575,7 @@ fwd32_kernel(const KP32 *__restrict__ kpg, const float *__restrict__ u, const fl
              float *__restrict__ pcost, JLog<float, D32> jl, int *__restrict__ jcnt, int *status,
              int64_t mloc, const __grid_constant__ RoundKeys rk) {
   constexpr bool SPLIT = TC == 2;
-  __shared__ __align__(1024) TcShared sh;
+  __shared__ __align__(1024) TcShared<SPLIT> sh;
   __shared__ __align__(16) CcShared cs;
   __shared__ __align__(16) float vbuf[32 * TPB];   // product staging (CUDA cores, jump steps)
   __shared__ Pair<float> red[TPB / 32];
@@ -466,10 +595,8 @@ fwd32_kernel(const KP32 *__restrict__ kpg, const float *__restrict__ u, const fl
   for (int c = 0; c < 32; ++c) x[c] = kp.x0[c];
   Kahan<float> cost;
   uint32_t fw = 0;
-  LogWriter<float, D32> lw;
-  lw.L = jl;
-  lw.idx = lm;
-  if (!active || !store) lw.L.cap = 0;
+  int nrec = 0;   // log records of the path
+  const int cap = active && store ? jl.cap : 0;
 #pragma unroll 1
   for (int k = 0; k <= Nt; ++k) {
     if (store && active) {
@@ -503,33 +630,20 @@ fwd32_kernel(const KP32 *__restrict__ kpg, const float *__restrict__ u, const fl
     }
     const unsigned om = __ballot_sync(0xffffffffu, one);   // every lane of the warp is in the loop
     if (__builtin_expect(om != 0u, 0)) {
-      float y1[32];
-      const float th = coop_one_jumps(kp, cs.at, vbuf + (threadIdx.x & ~31u), k, m, u, om, x, f, y1);
+      coop_one_jumps(kp, cs.at, vbuf + (threadIdx.x & ~31u), k, m, u, om, x, f, jl, lm, cap, nrec);
       if (one) {
         fw |= 1u << (k & 31);
-        if (lw.fits(1)) lw.put(k, 0, th, y1);
+        if (nrec + 1 <= cap) ++nrec;
       }
     }
-    if (jump && !one) {
-      // two or more jumps (rare): the generic routine on the CUDA cores (x is X_k)
-      fw |= 1u << (k & 31);
-      JumpStep<float, D32> S;
-      float zl[32], ul[DU32], xl[32];
-      (void)main_draws(kp, k, m, zl);
-#pragma unroll
-      for (int l = 0; l < DU32; ++l) ul[l] = __ldg(u + (size_t)k * DU32 + l);
-#pragma unroll
-      for (int c = 0; c < 32; ++c) xl[c] = x[c];
-      build_jump_step(kp, k, m, w0, zl, ul, xl, &S);
-#pragma unroll
-      for (int c = 0; c < 32; ++c) x[c] = S.Y[S.n + 1][c];
-      if (lw.fits(S.n)) {
-        for (int i = 0; i < S.n; ++i) {
-          float y[32];
-#pragma unroll
-          for (int c = 0; c < 32; ++c) y[c] = S.Y[i + 1][c];
-          lw.put(k, i, S.th[i], y);
-        }
+    const unsigned mm = __ballot_sync(0xffffffffu, jump && !one);
+    if (__builtin_expect(mm != 0u, 0)) {
+      coop_jumps(kp, cs.at, vbuf + (threadIdx.x & ~31u), k, m, w0, u, mm, x, jl, lm, cap, nrec);
+      if (jump && !one) {
+        int n = 0;
+        for (int i = 0; i < NMAX; ++i) n += ((unsigned long long)w0 >= kp.thr[i]) ? 1 : 0;
+        fw |= 1u << (k & 31);
+        if (nrec + n <= cap) nrec += n;
       }
     }
     cost.add(cost_term(kp, x, xd + (size_t)(k + 1) * D32));
@@ -538,7 +652,7 @@ fwd32_kernel(const KP32 *__restrict__ kpg, const float *__restrict__ u, const fl
       fw = 0;
     }
   }
-  if (store && active) jcnt[lm] = lw.r;
+  if (store && active) jcnt[lm] = nrec;
   Pair<float> v = cost.pair();
   if (!active) v = {0.f, 0.f};
   if (pcost && active) pcost[lm] = v.s + v.e;
@@ -627,7 +741,7 @@ adj32_kernel(const KP32 *__restrict__ kpg, const float *__restrict__ u, const fl
              const int *__restrict__ jcnt, double *__restrict__ partG, float *__restrict__ lam_out,
              int *status, int64_t mloc) {
   constexpr bool SPLIT = TC == 2;
-  __shared__ __align__(1024) TcShared sh;
+  __shared__ __align__(1024) TcShared<SPLIT> sh;
   __shared__ __align__(16) CcShared cs;
   __shared__ __align__(16) float vbuf[32 * TPB];   // product staging (CUDA cores, jump sub-steps)
   stage_params(cs, kpg);
