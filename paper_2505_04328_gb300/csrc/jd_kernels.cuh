@@ -1415,9 +1415,10 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
 // by instruction issue: M = 2^20, N_t = 1000, lambda dt = 0.01 (double well), store sweep
 // 9.60 -> 8.57 ms.  Without jumps a step of the cost sweep takes 1.9 ms of Philox rounds, 2.1
 // of the Box-Muller transform and 1.7 of the rest (parts of the sweep left out, per 1000
-// steps); the jumps, 2.5 ms before, take about 1.5.  Records per path and chunk and the draws
-// loop's unrolling, measured: single sweeps 2 records (64 registers; 3: 72 and 1% slower),
-// unrolled twice (1% faster); the paired sweep 3 records, rolled (unrolled 15% slower).
+// steps); the jumps, 2.5 ms before, take about 1.5.  Records per path and chunk, measured:
+// single sweeps 2 (64 registers; 3: 72 and 1% slower), the paired sweep 3.  The draws loop
+// unrolled four times, with the branch-free transform (store 8.28 -> 8.19 ms, paired 3% and
+// checkpoint sweeps 3% faster than rolled or unrolled twice).
 template <typename R, int D, bool PAIR>
 struct __align__(16) FwdChunkSmem {
   static constexpr int ROWS = FwdChunk<R, D>::CH * D + (PAIR ? 3 : 2) * FwdChunk<R, D>::W;
@@ -1630,7 +1631,7 @@ fwd_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u
                                           second ? nullptr : jcnt, mloc, PairOut<R, D>{}, pd1, red);
   } else if constexpr (CHUNK) {
     __shared__ FwdChunkSmem<R, D, PAIR> sm;
-    fwd_chunk_body<R, D, DU, MODE, PAIR, true, PAIR ? 1 : 2>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt,
+    fwd_chunk_body<R, D, DU, MODE, PAIR, true, 4>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt,
                                                mloc, p2, sm, red);
   } else {
     fwd_body<R, D, DU, MODE, PAIR, PRE, RK>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt, mloc,
@@ -2005,7 +2006,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
       for (int c0 = 0; c0 < len; c0 += kp.chunk) {
         const int clen = min(kp.chunk, len - c0);
         R(*const col)[TPB] = reinterpret_cast<R(*)[TPB]>(sbuf + (size_t)c0 * D * TPB);
-        const ChunkBits cb = chunk_draws<R, D, DU, 1, true>(kp, k0 + c0, clen, m, col, srec, RCREC);
+        const ChunkBits cb = chunk_draws<R, D, DU, 4, true>(kp, k0 + c0, clen, m, col, srec, RCREC);
         jm |= (uint64_t)cb.jump << c0;
         int rr = 0;
 #pragma unroll 1
@@ -2121,8 +2122,9 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
 // probability 6e-4.  Bound by instruction issue.  Before, the replay drew a jump step's slot
 // in divergent code per step and the backward regenerated every jump step through
 // jump_backward: 39.1 -> 13.8 ms per launch at M = 2^20, N_t = 1024, lambda dt = 0.0098 (27%
-// of the warp-steps have a jump).  The draws loop rolled, with the round keys from the
-// parameter block (unrolled 2 or 4 times 13.8 / 13.9 ms; keys bumped 14.1 ms).
+// of the warp-steps have a jump).  The draws loop unrolled twice, with the round keys from
+// the parameter block (13.3 ms with the branch-free transform; rolled 13.55, unrolled 4 or 8
+// times 13.5 / 16.4).
 template <typename R, int D>
 struct ThetaRecs {
   static constexpr int N = 2;             // records per path and segment
@@ -2204,7 +2206,7 @@ __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, cons
     for (int c = 0; c < D; ++c) x[c] = __ldg(ckpt + ((size_t)seg * D + c) * mloc + lmc);
     // bit i: step k0 + i had jumps (jm); exactly one (om1) (S <= 64)
     uint64_t jm = 0, om1 = 0;
-#pragma unroll 1
+#pragma unroll 2
     for (int i = 0; i < len; ++i) {
       R z[D];
       const uint32_t w0 = main_draws<true>(kp, k0 + i, m, z);

@@ -1,4 +1,4 @@
-"""The double-precision normals of the generator against extended precision."""
+"""The normals of the generator against extended precision."""
 import numpy as np
 import pytest
 
@@ -19,17 +19,19 @@ def _philox(c, key):
     return c
 
 
+@pytest.mark.parametrize("prec,tol", [("fp64", 2.5 * 2.0 ** -52), ("fp32", 4 * 2.0 ** -23)])
 @pytest.mark.parametrize("seed", [0, 5, (7 << 32) + 1])
-def test_normals_of_one_step(seed):
+def test_normals_of_one_step(seed, prec, tol):
     """One step of length 1 from 0 with unit noise and no drift is the step's normal pair.
-    Radius and cosine are within 0.86 and 1.0 units of the last place and the product rounds
-    once: below 2.5 units, 2.5 x 2^-52 of the value."""
+    FP64: radius and cosine are within 0.86 and 1.0 units of the last place and the product
+    rounds once: below 2.5 units, 2.5 x 2^-52 of the value.  FP32: the library's logarithm
+    (1 unit, halved by the root), root (0.5), sincospi (2) and product (0.5): 4 units."""
     build()
     M = 1 << 16
     p = workloads.ks_oscillator(M=M, Nt=1).replace(
         T=1.0, A=np.zeros((2, 2)), B=np.zeros((2, 1)), sigma=np.ones(2), x0=np.zeros(2), lam=0.0,
         xd=np.zeros((2, 2)), seed=seed)
-    with JdProblem(p, prec="fp64") as jp:
+    with JdProblem(p, prec=prec) as jp:
         X, _, _ = jp.sample_paths(np.zeros((1, 1)), 0, M, lam=False)
     m = np.arange(M, dtype=np.uint64)
     w = _philox([0 * m, m, 0 * m, 0 * m], seed)
@@ -42,4 +44,4 @@ def test_normals_of_one_step(seed):
     c, s = np.cos(a), np.sin(a)
     r = np.sqrt(-2 * np.log(u[0]))
     z = np.stack([r * np.choose(q, [c, -s, -c, s]), r * np.choose(q, [s, c, -s, -c])], axis=1)
-    assert np.max(np.abs((X[:, 1, :] - z) / z)) <= 2.5 * 2.0 ** -52
+    assert np.max(np.abs((X[:, 1, :] - z) / z)) <= tol
