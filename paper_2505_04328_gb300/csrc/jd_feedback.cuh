@@ -116,6 +116,11 @@ struct RingX {
       par ^= 1;
     }
   }
+  // A block of a cluster stays until its neighbours have read its buffer: a block that
+  // leaves after the last exchange takes its shared memory with it.
+  __device__ __forceinline__ void finish() const {
+    if constexpr (RING == 3) cooperative_groups::this_cluster().sync();
+  }
 };
 
 
@@ -480,6 +485,7 @@ fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
   }
   const double bs = fb_block_sum(active ? cost.pair() : Pair<R>{R(0), R(0)}, red);
   if (threadIdx.x == 0) partC[blockIdx.x] = bs;
+  rx.finish();
 }
 
 // 32-path dot products of a 2 x 2 block of weights: pa is the pair row of rows i, i+1 of
@@ -708,6 +714,7 @@ fb_adj_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
     }
     fb_store_partial<R, NX, NV>(partW + ((size_t)wid * Nt + k) * LP, lane, sq);
   }
+  rx.finish();
 }
 
 // ---------------------------------------------------------------------------
