@@ -487,10 +487,30 @@ static void free_dev(const jd_problem *p, T *&ptr) {
   ptr = nullptr;
 }
 
+// The feedback sweep's jump log is optional (without it the adjoint regenerates the jump
+// steps): an allocation that finds no room takes its memory.
+static void drop_fb_log(jd_problem *p) {
+  free_dev(p, p->fb_log_kt);
+  free_dev(p, p->fb_log_y);
+  free_dev(p, p->fb_jcnt);
+  p->bytes -= p->fb_log_bytes;
+  p->fb_log_bytes = 0;
+  p->fb_log_cap = 0;
+  p->fb_log_state = -1;
+}
+// Device bytes in use besides the droppable log.
+static size_t held_bytes(const jd_problem *p) { return p->bytes - p->fb_log_bytes; }
+
 static jd_status dev_alloc(jd_problem *p, void **ptr, size_t bytes, const char *what) {
+  if (p->bytes + bytes > p->budget && p->fb_log_bytes) drop_fb_log(p);
   if (p->bytes + bytes > p->budget)
     return fail(JD_ERR_OOM, std::string("memory budget exceeded allocating ") + what);
   cudaError_t e = p->async_alloc ? cudaMallocAsync(ptr, bytes, p->stream) : cudaMalloc(ptr, bytes);
+  if (e != cudaSuccess && p->fb_log_bytes) {
+    cudaGetLastError();
+    drop_fb_log(p);
+    e = p->async_alloc ? cudaMallocAsync(ptr, bytes, p->stream) : cudaMalloc(ptr, bytes);
+  }
   if (e != cudaSuccess) {
     cudaGetLastError();
     return fail(JD_ERR_OOM, std::string("cudaMalloc failed for ") + what + ": " + cudaGetErrorString(e));
@@ -584,13 +604,13 @@ static jd_status ensure_plan(jd_problem *p) {
     want = JD_ADJ_STORED;
   }
   if (want == JD_ADJ_AUTO)
-    want = (p->bytes + stored_bytes(p) <= p->budget) ? JD_ADJ_STORED : JD_ADJ_RECOMPUTE;
+    want = (held_bytes(p) + stored_bytes(p) <= p->budget) ? JD_ADJ_STORED : JD_ADJ_RECOMPUTE;
   if (want == JD_ADJ_STORED) {
     int64_t M = p->desc.M;
-    if (p->D == 32 && p->bytes + stored_bytes(p) > p->budget) {
+    if (p->D == 32 && held_bytes(p) + stored_bytes(p) > p->budget) {
       // no recompute adjoint at d = 32: store the paths block by block, the largest
       // multiple of 128 paths whose states fit what is left of the budget
-      const size_t avail = p->budget > p->bytes ? p->budget - p->bytes : 0;
+      const size_t avail = p->budget > held_bytes(p) ? p->budget - held_bytes(p) : 0;
       const size_t per128 = stored_plan_bytes(p->desc, p->D, elem_size(p), TPB);
       int64_t c = (int64_t)(avail / per128) * TPB;
       while (c >= TPB && stored_plan_bytes(p->desc, p->D, elem_size(p), c) > avail) c -= TPB;
@@ -612,7 +632,7 @@ static jd_status ensure_plan(jd_problem *p) {
     s = dev_alloc(p, (void **)&p->jcnt, (size_t)M * 8, "jump log counts");
     if (s) return s;
   } else {
-    const size_t avail = p->budget > p->bytes ? p->budget - p->bytes : 0;
+    const size_t avail = p->budget > held_bytes(p) ? p->budget - held_bytes(p) : 0;
     const int S = choose_spacing(p, avail);
     if (!S) return fail(JD_ERR_OOM, "the memory budget does not hold the checkpoints of the recompute plan");
     p->S = S;
@@ -732,7 +752,7 @@ static bool ensure_pair(jd_problem *p) {
   const bool stored = p->plan == JD_ADJ_STORED;
   const size_t cap = (size_t)(p->log_cap > 0 ? p->log_cap : 1);
   const size_t b_traj = traj_values(q.Nt, p->D, (int)es, (int64_t)M) * es;
-  if (p->bytes + jd::pair_bytes(q, p->plan) > p->budget) return false;
+  if (held_bytes(p) + jd::pair_bytes(q, p->plan) > p->budget) return false;
   const std::string saved_error = g_last_error;   // a failed allocation here is not the caller's error
   jd_status s = dev_alloc(p, &p->uk2, (size_t)q.Nt * p->DU * es, "paired control");
   if (!s) s = dev_alloc(p, (void **)&p->partC2, (size_t)p->nblk * 8, "paired cost partials");
@@ -1439,6 +1459,7 @@ jd_status jd_problem_destroy(jd_problem *p) {
   free_dev(p, p->fb_partC);
   free_dev(p, p->fb_partG);
   free_dev(p, p->fb_partW);
+  drop_fb_log(p);
   free_dev(p, p->fb_mut);
   if (p->host_pinned && p->own_pinned) cudaFreeHost(p->host_pinned);
   if (p->own_stream && p->stream) cudaStreamDestroy(p->stream);
@@ -2018,6 +2039,23 @@ static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad) {
     s = dev_alloc(p, (void **)&p->fb_partG, (size_t)fb_groups(nwarp) * Nt * LP * 8, "feedback group partials");
   if (!s && !p->fb_z0) s = dev_alloc(p, &p->fb_z0, (size_t)2 * RING_MAX * es, "ring initial states");
   if (s) return s;
+  if (grad && p->fb_log_state == 0) {   // last, and only where there is room
+    const int cap = log_capacity(p->desc);
+    const size_t nk = (size_t)cap * M * 2 * es, nb = 2 * nk + (size_t)M * 8;
+    p->fb_log_state = -1;
+    if (cap > 0 && p->bytes + nb <= p->budget) {
+      if (cudaMalloc(&p->fb_log_kt, nk) == cudaSuccess && cudaMalloc(&p->fb_log_y, nk) == cudaSuccess &&
+          cudaMalloc((void **)&p->fb_jcnt, (size_t)M * 8) == cudaSuccess) {
+        p->fb_log_bytes = nb;
+        p->bytes += nb;
+        p->fb_log_cap = cap;
+        p->fb_log_state = 1;
+      } else {
+        cudaGetLastError();
+        drop_fb_log(p);
+      }
+    }
+  }
   // once per padded size: raising the limit reallocates local memory (a device-wide sync)
   const size_t need = ops->stack_bytes();
   if (need > p->fb_stack) {
@@ -2063,6 +2101,10 @@ static jd_status fb_run(jd_problem *p, const jd_feedback_desc *fb, const double 
   b.mu = p->fb_mu;
   b.traj = p->fb_traj;
   b.flags = p->fb_flags;
+  b.log_kt = p->fb_log_kt;
+  b.log_y = p->fb_log_y;
+  b.jcnt = p->fb_jcnt;
+  b.log_cap = p->fb_log_cap;
   b.partC = p->fb_partC;
   b.partW = p->fb_partW;
   b.partG = p->fb_partG;

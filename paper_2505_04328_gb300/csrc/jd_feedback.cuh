@@ -29,6 +29,12 @@
 // The kernels work on padded sizes NX x NV (instances 4x4, 10x10, 16x16): the weights
 // beyond nx x nv are 0, so the bumps of the padding centres do not reach u.
 //
+// The forward that keeps states for the adjoint logs the post-jump states too (the jump log of
+// the path kernels, where the memory budget holds it), so the adjoint regenerates only what
+// the log does not hold: 5.55 -> 4.30 ms at M = 2^20, N_t = 100, lambda dt = 0.018 (3.4
+// without jumps); the forward takes a one-jump step's draws in straight code, 2.99 -> 2.56 ms
+// (1.7 without jumps).
+//
 // A step with jumps runs its sub-steps in the same loop as a step without (forward: one
 // sub-step per iteration; adjoint: one backward sub-step and one warp exchange per
 // round), so a warp in which one path jumps pays one more pass of the same code rather
@@ -405,11 +411,23 @@ __device__ __forceinline__ double fb_block_sum(Pair<R> v, Pair<R> *red) {
   return out;
 }
 
+// Resident blocks per SM asked of the compiler (its own choice took 98 registers forward and
+// 230 in the adjoint with the jump log): FP32 10 x 10 forward 3 blocks of 80 registers 2.56 ms,
+// unbounded 3.64 (M = 2^20, N_t = 100); adjoint 2 blocks of 128 4.30, unbounded 5.35, 3 of 80
+// 4.90.
+template <typename R, int NX, int NV>
+constexpr int fb_fwd_blocks() {
+  return sizeof(R) == 8 || NX * NV > 100 ? 2 : 3;
+}
+template <typename R, int NX, int NV>
+constexpr int fb_adj_blocks() {
+  return sizeof(R) == 8 ? 1 : NX * NV <= 16 ? 3 : 2;
+}
 template <typename R, int NX, int NV, bool STORE, int RING>
-__global__ void __launch_bounds__(FB_TPB)
+__global__ void __launch_bounds__(FB_TPB, fb_fwd_blocks<R, NX, NV>())
 fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant__ FbParams<R> fp,
               const R *__restrict__ mu, const R *__restrict__ xd, R *__restrict__ traj,
-              uint32_t *__restrict__ flags, double *__restrict__ partC) {
+              uint32_t *__restrict__ flags, JLog<R, 2> jl, int *__restrict__ jcnt, double *__restrict__ partC) {
   using M = Ar<R>;
   constexpr int LP = NX * NV;
   constexpr bool CPL = RING > 0;
@@ -434,6 +452,10 @@ fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
       z[1] = fp.z0[fp.S + rx.i];
     }
     uint32_t fw = 0;
+    LogWriter<R, 2> lw;   // post-jump states for the adjoint
+    lw.L = jl;
+    lw.idx = m;
+    if (!STORE || !active || !jcnt) lw.L.cap = 0;
     if (STORE && active) {
       traj[m] = z[0];
       traj[mloc + m] = z[1];
@@ -452,9 +474,20 @@ fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
       const uint32_t w0 = main_draws<true>(kp, k, mg, zs);   // round keys of the parameter block
       int n = 0;
       FbPlan<R> P;
+      // a step with one jump takes its slot's draws in straight code, any other jump step the
+      // plan's loops
+      bool one = false, log = false;
+      R th1 = R(1), xih1[2] = {R(0), R(0)}, z1[2] = {R(0), R(0)};
       if (has_jump(kp, w0)) {
-        n = fb_plan(kp, k, mg, w0, P);
+        one = (unsigned long long)w0 < kp.thr[1];
+        if (one) {
+          n = 1;
+          th1 = slot_draws_at<true>(kp, k, mg, 0, xih1, z1);
+        } else {
+          n = fb_plan(kp, k, mg, w0, P);
+        }
         fw |= 1u << (k & 31);
+        if (STORE) log = lw.take(n, k);
       }
       // sub-steps 0..n (one when the step has no jump) in one loop, so that a warp with
       // a jumping path runs the same code for every sub-step (Algorithm 5.1)
@@ -462,14 +495,20 @@ fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
       for (int i = 0;; ++i) {
         R de = kp.dt, sq = kp.sqdt;
         if (n > 0) {
-          de = fb_delta(kp, P, n, i);
+          de = one ? M::mul(kp.dt, i == 0 ? th1 : M::sub(R(1), th1)) : fb_delta(kp, P, n, i);
           sq = Ar<R>::sqrt(de);
         }
         cost.add(fb_substep<R, NX, NV, CPL>(kp, fp, mk, de, sq, zs, z, cin));
         if (i >= n) break;
-        R xih[2];
-        slot_draws(kp, k, mg, P.order[i], xih, zs);   // the jump's size and the next normals
+        R xih[2] = {xih1[0], xih1[1]};   // the jump's size and the next normals
+        if (one) {
+          zs[0] = z1[0];
+          zs[1] = z1[1];
+        } else {
+          slot_draws(kp, k, mg, P.order[i], xih, zs);
+        }
         apply_jump(kp, z, xih);
+        if (STORE && log) lw.put(k, i, one ? th1 : P.th[i], z);
       }
       R g[2];
       cost.add(fb_track<R, false>(fp, kp.dt, z, xd + (size_t)(k + 1) * 2, g));
@@ -481,6 +520,10 @@ fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
           fw = 0;
         }
       }
+    }
+    if (STORE && active && jcnt) {
+      jcnt[m] = lw.r;
+      jcnt[mloc + m] = min(lw.kovf, Nt);
     }
   }
   const double bs = fb_block_sum(active ? cost.pair() : Pair<R>{R(0), R(0)}, red);
@@ -583,10 +626,11 @@ constexpr size_t fb_adj_smem() {
 }
 
 template <typename R, int NX, int NV, int RING>
-__global__ void __launch_bounds__(FB_TPB)
+__global__ void __launch_bounds__(FB_TPB, fb_adj_blocks<R, NX, NV>())
 fb_adj_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant__ FbParams<R> fp,
               const R *__restrict__ mu, const R *__restrict__ xd, const R *__restrict__ traj,
-              const uint32_t *__restrict__ flags, R *__restrict__ partW) {
+              const uint32_t *__restrict__ flags, JLog<R, 2> jl, const int *__restrict__ jcnt,
+              R *__restrict__ partW) {
   using M = Ar<R>;
   constexpr int LP = NX * NV, QPL = fb_qpl<NX, NV>();   // 2 x 2 blocks per lane
   constexpr bool CPL = RING > 0;
@@ -620,6 +664,10 @@ fb_adj_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
     zn[1] = traj[((size_t)(Nt - 1) * 2 + 1) * mloc + m];
     fword = flags[(size_t)((Nt - 1) >> 5) * mloc + m];
   }
+  // the log holds every jump step before kovf (0: no log)
+  LogReader2<R, 2> lr;
+  lr.init(jl, m, active && jcnt ? min(__ldg(jcnt + m), jl.cap) : 0);
+  const int kovf = active && jcnt ? __ldg(jcnt + mloc + m) : 0;
 #pragma unroll 1
   for (int k = Nt - 1; k >= 0; --k) {
     const R *mk = mu + (size_t)k * LP;
@@ -642,7 +690,10 @@ fb_adj_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
       if (active)
         cin = M::mul(fp.omega, M::add(traj[((size_t)k * 2) * mloc + mleft], traj[((size_t)k * 2) * mloc + mright]));
     }
-    if (active) {
+    const bool logged = active && ((fk >> (k & 31)) & 1u) && k < kovf;
+    if (logged) n = lr.ci + 1;   // the step's last record is the reader's current one
+    R thn = R(1);
+    if (active && !logged) {
       if ((fk >> (k & 31)) & 1u) {
         // regenerate the step's sub-states from X_k with the forward's arithmetic
         R zs[2], y[2] = {zk[0], zk[1]};
@@ -676,7 +727,12 @@ fb_adj_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
         if (i < n) jump_adjoint(kp, a);   // across the jump that ends sub-step i
         R y[2] = {zk[0], zk[1]};
         R de = kp.dt;
-        if (n > 0) {
+        if (logged) {   // fb_delta from the records' times
+          R th = R(0);
+          if (i > 0) lr.pop(th, y);
+          de = M::mul(kp.dt, M::sub(thn, th));
+          thn = th;
+        } else if (n > 0) {
           de = fb_delta(kp, P, n, i);
           if (i > 0) {
             y[0] = Ys[i][0];
@@ -988,11 +1044,17 @@ cudaError_t fb_launch(void (*kern)(KArgs...), int ring, int S, unsigned grid, si
   return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+template <typename R>
+JLog<R, 2> fb_log(const FbBufs &b, int64_t mloc) {
+  return JLog<R, 2>{static_cast<typename V2<R>::T *>(b.log_kt), static_cast<R *>(b.log_y), mloc, b.log_cap};
+}
+
 template <typename R, int NX, int NV, bool STORE, int RING>
-cudaError_t fb_fwd_ring(const KParams<R, 2, 1> &kp, const FbParams<R> &fp, const R *mu, const R *xd, R *traj,
-                        uint32_t *flags, double *partC, unsigned grid, cudaStream_t s) {
-  return fb_launch(fb_fwd_kernel<R, NX, NV, STORE, RING>, RING, fp.S, grid, 0, s, kp, fp, mu, xd, traj, flags,
-                   partC);
+cudaError_t fb_fwd_ring(const KParams<R, 2, 1> &kp, const FbParams<R> &fp, const R *mu, const R *xd, const FbBufs &b,
+                        unsigned grid, cudaStream_t s) {
+  return fb_launch(fb_fwd_kernel<R, NX, NV, STORE, RING>, RING, fp.S, grid, 0, s, kp, fp, mu, xd,
+                   STORE ? static_cast<R *>(b.traj) : nullptr, STORE ? b.flags : nullptr, fb_log<R>(b, fp.mloc),
+                   STORE ? b.jcnt : nullptr, b.partC);
 }
 
 template <typename R, int NX, int NV>
@@ -1004,17 +1066,15 @@ cudaError_t fb_fwd_launch(const ::jd_problem *p, const jd_feedback_desc &fb, boo
   fb_make_params<R>(p, fb, fp);
   const unsigned grid = (unsigned)ceil_div(p->desc.M, FB_TPB);
   const R *mu = static_cast<const R *>(b.mu), *xd = static_cast<const R *>(p->xdk);
-  R *traj = store ? static_cast<R *>(b.traj) : nullptr;
-  uint32_t *flags = store ? b.flags : nullptr;
   switch (ring_kind(fb.particles) * 2 + (store ? 1 : 0)) {
-    case 0: return fb_fwd_ring<R, NX, NV, false, 0>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
-    case 1: return fb_fwd_ring<R, NX, NV, true, 0>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
-    case 2: return fb_fwd_ring<R, NX, NV, false, 1>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
-    case 3: return fb_fwd_ring<R, NX, NV, true, 1>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
-    case 4: return fb_fwd_ring<R, NX, NV, false, 2>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
-    case 5: return fb_fwd_ring<R, NX, NV, true, 2>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
-    case 6: return fb_fwd_ring<R, NX, NV, false, 3>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
-    default: return fb_fwd_ring<R, NX, NV, true, 3>(kp, fp, mu, xd, traj, flags, b.partC, grid, s);
+    case 0: return fb_fwd_ring<R, NX, NV, false, 0>(kp, fp, mu, xd, b, grid, s);
+    case 1: return fb_fwd_ring<R, NX, NV, true, 0>(kp, fp, mu, xd, b, grid, s);
+    case 2: return fb_fwd_ring<R, NX, NV, false, 1>(kp, fp, mu, xd, b, grid, s);
+    case 3: return fb_fwd_ring<R, NX, NV, true, 1>(kp, fp, mu, xd, b, grid, s);
+    case 4: return fb_fwd_ring<R, NX, NV, false, 2>(kp, fp, mu, xd, b, grid, s);
+    case 5: return fb_fwd_ring<R, NX, NV, true, 2>(kp, fp, mu, xd, b, grid, s);
+    case 6: return fb_fwd_ring<R, NX, NV, false, 3>(kp, fp, mu, xd, b, grid, s);
+    default: return fb_fwd_ring<R, NX, NV, true, 3>(kp, fp, mu, xd, b, grid, s);
   }
 }
 
@@ -1027,7 +1087,8 @@ cudaError_t fb_adj_ring(const KParams<R, 2, 1> &kp, const FbParams<R> &fp, const
   if (e != cudaSuccess) return e;
   return fb_launch(fb_adj_kernel<R, NX, NV, RING>, RING, fp.S, grid, smem, s, kp, fp,
                    static_cast<const R *>(b.mu), xd, static_cast<const R *>(b.traj),
-                   static_cast<const uint32_t *>(b.flags), static_cast<R *>(b.partW));
+                   static_cast<const uint32_t *>(b.flags), fb_log<R>(b, fp.mloc), static_cast<const int *>(b.jcnt),
+                   static_cast<R *>(b.partW));
 }
 
 // The adjoint sweep (warp partials of the gradient).

@@ -168,6 +168,9 @@ struct FbBufs {
   const void *mu = nullptr;     // [Nt][NX/2][NV][2] padded, interleaved weights, kernel precision
   void *traj = nullptr;         // [Nt+1][2][M] states (gradient only)
   uint32_t *flags = nullptr;    // [ceil(Nt/32)][M] jump flags (gradient only)
+  void *log_kt = nullptr, *log_y = nullptr;   // jump log (gradient, where the budget holds it)
+  int *jcnt = nullptr;          // its counts and closing steps; null: no log
+  int log_cap = 0;
   double *partC = nullptr;      // [nblk] cost partials
   void *partW = nullptr;        // [nwarp][Nt][NX*NV] warp partials, kernel precision
   double *partG = nullptr;      // [ngroup][Nt][NX*NV] FP64 group partials
@@ -282,6 +285,12 @@ struct jd_problem {
   uint32_t *fb_flags = nullptr;
   double *fb_mu64 = nullptr, *fb_grad = nullptr, *fb_partC = nullptr, *fb_partG = nullptr;
   void *fb_partW = nullptr;
+  // post-jump states of the feedback sweep for its adjoint, kept while the budget has room
+  // (dev_alloc drops them first); fb_log_state: 0 not tried, 1 there, -1 without
+  void *fb_log_kt = nullptr, *fb_log_y = nullptr;
+  int *fb_jcnt = nullptr;
+  int fb_log_cap = 0, fb_log_state = 0;
+  size_t fb_log_bytes = 0;
   void *fb_z0 = nullptr;     // interacting particles: the ring's initial states [2][S], kernel precision
   double *fb_mut = nullptr;  // optimizer: trial weights (FP64)
   int fb_LP = 0;             // padded weights per step of fb_mu / fb_partW / fb_partG

@@ -245,3 +245,37 @@ def test_optimizer_reuses_the_accepted_trial_sweep():
         _, rs, _ = jp.fb_optimize(fb.replace(adjoint=workloads.FB_SURROGATE, sur_rate=0.05), max_iter=3,
                                   tol_rel_grad=0.0)
         assert rs["sweeps"] == rs["evals"]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("lam", [1.78, 40.0, 400.0])
+def test_adjoint_with_and_without_the_jump_log(prec, lam):
+    """The jump log is kept where the memory budget has room for it; without it the adjoint
+    regenerates every jump step: the same operations, so the same bits.  A budget that holds
+    everything but the log gives the form without."""
+    p, fb = workloads.feedback_centering(M=3000, Nt=45)
+    p = p.replace(lam=lam)
+    mu = workloads.random_mu(p, fb, seed=5, scale=0.4)
+    with JdProblem(p, prec=prec) as jp:
+        J, g = jp.fb_gradient(fb, mu)
+        full = jp.info()["device_bytes"]
+    with JdProblem(p, prec=prec, mem_budget=full - 8) as jp:
+        J0, g0 = jp.fb_gradient(fb, mu)
+        assert jp.info()["device_bytes"] < full
+    assert J == J0 and np.array_equal(g, g0)
+
+
+def test_the_jump_log_gives_way_to_other_allocations():
+    """A later allocation that finds no room takes the log's memory."""
+    p, fb = workloads.feedback_centering(M=4096, Nt=40)
+    mu = workloads.random_mu(p, fb, seed=6, scale=0.4)
+    with JdProblem(p) as jp:
+        J, g = jp.fb_gradient(fb, mu)
+        with_log = jp.info()["device_bytes"]
+    u = np.zeros((p.Nt, 1))
+    with JdProblem(p, mode="recompute", mem_budget=with_log + 1000) as jp:
+        assert np.array_equal(jp.fb_gradient(fb, mu)[1], g)
+        jp.gradient(u)                              # needs the checkpoints' memory
+        assert jp.info()["device_bytes"] <= with_log + 1000
+        J1, g1 = jp.fb_gradient(fb, mu)
+    assert J1 == J and np.array_equal(g1, g)
