@@ -81,7 +81,7 @@ static cudaError_t op32_adj(const jd_problem *p, int variant, bool theta, int64_
   return cudaGetLastError();
 }
 
-static size_t op32_stack() {
+static size_t query32_stack() {
   size_t need = 4 * sizeof(JumpStep<float, D32>) + 2048;   // >= the cumulative frames reported by ptxas
   const void *ks[] = {(const void *)fwd32_kernel<0>, (const void *)fwd32_kernel<1>, (const void *)fwd32_kernel<2>,
                       (const void *)adj32_kernel<0>, (const void *)adj32_kernel<1>, (const void *)adj32_kernel<2>};
@@ -90,6 +90,11 @@ static size_t op32_stack() {
     if (cudaFuncGetAttributes(&a, k) == cudaSuccess && a.localSizeBytes + 1024 > need) need = a.localSizeBytes + 1024;
   }
   return (need + 255) & ~(size_t)255;
+}
+
+static size_t op32_stack() {   // asked once: the kernels' attributes do not change
+  static const size_t bytes = query32_stack();
+  return bytes;
 }
 
 extern const PathOps ops_f32_d32_u4 = PathOps{D32, DU32, 8, 4, 1, &op32_stack, &op32_fwd, &op32_adj, nullptr,

@@ -1253,6 +1253,41 @@ struct PreDraws {
   unsigned long long *held, key;   // the sweep records that the buffers hold the draws of key
 };
 
+// The pre-drawn sweep's inputs of the next N steps (draws, control, target row), copied to
+// shared memory ahead of their use: with four paths to a warp and a warp to an SM nothing else
+// hides a load's latency, and a step waited for its draws, its control and its target row in
+// turn.  Each thread copies and waits for its own values.  d = 1, N_t = 200, lambda dt = 0.01:
+// FP32 M = 1000 83 -> 58 us per sweep, M = 8000 89 -> 79; FP64 M = 1000, N_t = 100 122 -> 109
+// (FP64 arithmetic's latency remains).  A prefetch of one step in registers gave 116; copying
+// the slot draws of every step as well (few are used) 64 / 90 / 110.
+template <typename R, int D, int DU>
+struct PreRing {
+  static constexpr int N = 16;
+  R z[N][D][SPREAD_LANES], x[N][D][SPREAD_LANES], u[N][DU][SPREAD_LANES];
+  uint32_t w[N][SPREAD_LANES];
+  template <int B>
+  static __device__ __forceinline__ void copy(void *smem, const void *gmem) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], %2;\n" ::"r"((unsigned)__cvta_generic_to_shared(smem)),
+                 "l"(gmem), "n"(B)
+                 : "memory");
+  }
+  __device__ __forceinline__ void issue(const PreDraws<R, D> &pd, const R *__restrict__ uk, const R *__restrict__ xd,
+                                        int k, int Nt, int64_t mloc, int64_t lm) {
+    const int i = k & (N - 1), t = threadIdx.x;
+    if (k < Nt) {
+      copy<4>(&w[i][t], pd.w + (int64_t)k * mloc + lm);
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        copy<sizeof(R)>(&z[i][c][t], pd.z + ((int64_t)k * D + c) * mloc + lm);
+        copy<sizeof(R)>(&x[i][c][t], xd + (size_t)(k + 1) * D + c);
+      }
+#pragma unroll
+      for (int l = 0; l < DU; ++l) copy<sizeof(R)>(&u[i][l][t], uk + (size_t)k * DU + l);
+    }
+    cp_async_commit();   // an empty group past the end keeps the count uniform
+  }
+};
+
 // A step with one jump, its slot draws pre-drawn: sub-step to the jump, jump, sub-step.
 template <typename R, int D, int DU, typename LW>
 __device__ __forceinline__ void one_jump_pre(const KParams<R, D, DU> &kp, int k, const R *__restrict__ sk,
@@ -1284,7 +1319,8 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
                                          const R *__restrict__ xd, double *__restrict__ partC, R *__restrict__ traj,
                                          uint32_t *__restrict__ flags, R *__restrict__ ckpt, R *__restrict__ pcost,
                                          const JLog<R, D> &jl, int *__restrict__ jcnt, int64_t mloc,
-                                         const PairOut<R, D> &p2, const PreDraws<R, D> &pd, Pair<R> *red) {
+                                         const PairOut<R, D> &p2, const PreDraws<R, D> &pd, Pair<R> *red,
+                                         PreRing<R, D, DU> *ring = nullptr) {
   if (PRE && threadIdx.x >= SPREAD_LANES) return;   // no warp-wide operation follows in this mode
   const int64_t lm = PRE ? bid * SPREAD_LANES + threadIdx.x : bid * TPB + threadIdx.x;
   const bool active = lm < mloc;
@@ -1321,6 +1357,9 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
   for (int i = 0; i < StageBuf<R, D>::N; ++i)
 #pragma unroll
     for (int c = 0; c < D; ++c) sb.v[i][c] = sb2.v[i][c] = R(0);
+  if constexpr (PRE) {
+    for (int k = 0; k < ring->N - 1; ++k) ring->issue(pd, u, xd, k, Nt, mloc, active ? lm : 0);
+  }
   constexpr int UNR = ((PAIR || MODE == FWD_CKPT) && D <= 2) ? 2 : 1;
 #pragma unroll UNR
   for (int k = 0; k <= Nt; ++k) {
@@ -1337,16 +1376,22 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
       }
     }
     int nj;
+    R xk[D];
     if constexpr (PRE) {   // inactive threads read path 0's draws
-      const int64_t lmc = active ? lm : 0, ik = (int64_t)k * mloc + lmc;
-      const uint32_t w0 = pd.w[ik];
-      R z[D];
+      const int64_t lmc = active ? lm : 0;
+      ring->issue(pd, u, xd, k + ring->N - 1, Nt, mloc, lmc);
+      cp_async_wait<PreRing<R, D, DU>::N - 1>();   // step k's values have landed
+      const int s = k & (ring->N - 1), t = threadIdx.x;
+      const uint32_t w0 = ring->w[s][t];
+      R z[D], uk[DU];
 #pragma unroll
-      for (int c = 0; c < D; ++c) z[c] = pd.z[((int64_t)k * D + c) * mloc + lmc];
+      for (int c = 0; c < D; ++c) {
+        z[c] = ring->z[s][c][t];
+        xk[c] = ring->x[s][c][t];
+      }
+#pragma unroll
+      for (int l = 0; l < DU; ++l) uk[l] = ring->u[s][l][t];
       const R *sk = pd.s + (int64_t)k * (1 + 2 * D) * mloc + lmc;
-      R uk[DU];
-#pragma unroll
-      for (int l = 0; l < DU; ++l) uk[l] = __ldg(u + (size_t)k * DU + l);
       if (has_jump(kp, w0) && one_jump(kp, w0)) {   // the common jump step, pre-drawn
         one_jump_pre(kp, k, sk, mloc, z, uk, x, lw);
         if constexpr (PAIR) {
@@ -1369,7 +1414,10 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
       nj = forward_step_h<R, D, DU, LW, false, true, KH, RK>(kp, kh, k, m, u, x, lw);
     }
     if (nj) fw |= 1u << (k & 31);
-    cost.add(cost_term(kh, x, xd + (size_t)(k + 1) * D));
+    if constexpr (PRE)
+      cost.add(cost_term_row(kh, x, xk));
+    else
+      cost.add(cost_term(kh, x, xd + (size_t)(k + 1) * D));
     if constexpr (PAIR) cost2.add(cost_term(kh, x2, xd + (size_t)(k + 1) * D));
     if (MODE == FWD_STORE && ((k & 31) == 31 || k == Nt - 1)) {
       if (active && (!PRE || flags)) flags[(size_t)(k >> 5) * mloc + lm] = fw;
@@ -1625,10 +1673,15 @@ fwd_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u
     const bool second = blockIdx.x >= nb;
     PreDraws<R, D> pd1 = pd;
     if (second) pd1.cw = pd.cw2;
+    __shared__ PreRing<R, D, DU> ring;
     fwd_body<R, D, DU, MODE, false, true, RK>(kp, second ? blockIdx.x - nb : blockIdx.x, second ? p2.u : u, xd, partC,
                                           second ? p2.traj : traj, second ? nullptr : flags,
                                           second ? p2.ckpt : ckpt, nullptr, second ? p2.jl : jl,
-                                          second ? nullptr : jcnt, mloc, PairOut<R, D>{}, pd1, red);
+                                          second ? nullptr : jcnt, mloc, PairOut<R, D>{}, pd1, red, &ring);
+  } else if constexpr (PRE) {
+    __shared__ PreRing<R, D, DU> ring;
+    fwd_body<R, D, DU, MODE, PAIR, PRE, RK>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt, mloc,
+                                            p2, pd, red, &ring);
   } else if constexpr (CHUNK) {
     __shared__ FwdChunkSmem<R, D, PAIR> sm;
     fwd_chunk_body<R, D, DU, MODE, PAIR, true, 4>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt,
@@ -2822,7 +2875,7 @@ constexpr bool batch_built() {
 }
 
 template <typename R, int D, int DU>
-size_t op_stack_bytes() {
+size_t query_stack_bytes() {
   size_t need = 2 * sizeof(JumpStep<R, D>) + 2048;
   const void *ks[] = {
       (const void *)fwd_form<R, D, DU, FWD_COST>(false), (const void *)fwd_form<R, D, DU, FWD_STORE>(false),
@@ -2856,6 +2909,14 @@ size_t op_stack_bytes() {
     }
   }
   return (need + 255) & ~(size_t)255;
+}
+
+// (asked once per process: the kernels' attributes do not change, and each query costs several
+// microseconds of every problem's creation)
+template <typename R, int D, int DU>
+size_t op_stack_bytes() {
+  static const size_t bytes = query_stack_bytes<R, D, DU>();
+  return bytes;
 }
 
 template <typename R, int D, int DU>
