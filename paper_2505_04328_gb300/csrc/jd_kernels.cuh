@@ -321,6 +321,56 @@ __device__ __forceinline__ void one_jump_inline(const KParams<R, D, DU> &kp, int
   euler_substep(kp, M::mul(kp.dt, M::sub(R(1), th)), z1, uk, x);
 }
 
+// Slot-0 draws of the lanes of om, by the whole warp, for d > 2: a lane alone draws up to 5
+// Philox blocks and 8 Box-Muller pairs in divergent code; here, per jump lane, each block and
+// each pair is one lane's, and the lane takes its values from shared memory.  The values are
+// slot0_draws', so the same bits.  sc: this warp's scratch (SlotScratch).  Called by every lane
+// of the warp; th, xih, z1 are set in the lanes of om.  Where it pays: coop_slots.
+template <typename R, int D>
+struct __align__(16) SlotScratch {
+  static constexpr int PD = MainWords<D>::PD, NB = (1 + 4 * PD + 3) / 4;
+  uint4 w[NB];
+  R v[4 * PD];
+};
+template <typename R, int D, int DU>
+__device__ __forceinline__ void coop_slot0_draws(const KParams<R, D, DU> &kp, SlotScratch<R, D> &sc, int k, uint32_t m,
+                                                 unsigned om, R &th, R (&xih)[D], R (&z1)[D]) {
+  using M = Ar<R>;
+  constexpr int PD = SlotScratch<R, D>::PD, NB = SlotScratch<R, D>::NB;
+  const int lane = threadIdx.x & 31;
+  while (om) {
+    const int j = __ffs((int)om) - 1;
+    om &= om - 1;
+    const uint32_t mj = __shfl_sync(0xffffffffu, m, j);
+    if (lane < NB)
+      sc.w[lane] = philox10((uint32_t)k, mj, (1u << 24) | (1u << 16) | (uint32_t)lane, kp.epoch, kp.key0, kp.key1);
+    __syncwarp();
+    const uint32_t *w = reinterpret_cast<const uint32_t *>(sc.w);
+    if (lane < 2 * PD) {   // pairs 0 .. PD - 1: sizes; PD .. 2 PD - 1: the normals after the jump
+      const uint32_t wa = w[1 + 2 * lane], wb = w[2 + 2 * lane];
+      R a, b;
+      if (lane < PD && kp.jump_law == JD_JUMP_UNIFORM) {
+        a = M::sub(M::mul(R(2), M::u01(wa)), R(1));
+        b = M::sub(M::mul(R(2), M::u01(wb)), R(1));
+      } else {
+        normal_pair<R>(wa, wb, a, b);
+      }
+      sc.v[2 * lane] = a;
+      sc.v[2 * lane + 1] = b;
+    }
+    __syncwarp();
+    if (lane == j) {
+      th = M::u01(w[0]);
+#pragma unroll
+      for (int c = 0; c < D; ++c) {
+        xih[c] = c < kp.d ? sc.v[c] : R(0);
+        z1[c] = c < kp.d ? sc.v[2 * PD + c] : R(0);
+      }
+    }
+    __syncwarp();   // the scratch is the next lane's
+  }
+}
+
 // x <- x + dt f + sigma sqrt(dt) z: the step without jumps.
 template <typename KP, typename R, int D>
 __device__ __forceinline__ void plain_update(const KP &kp, const R (&f)[D], const R (&z)[D], R (&x)[D]) {
@@ -364,12 +414,24 @@ __device__ __forceinline__ void noisy_update(R de, const R (&f)[D], const R (&a)
 // (kp itself or a HotFwd); the jump paths read kp.  RK: the inline slot draws take the
 // round keys of kp (a __grid_constant__ parameter).
 template <typename R, int D, int DU, typename LW, bool INLINE_JUMP = true, typename KH = KParams<R, D, DU>,
-          bool RK = false>
+          bool RK = false, bool COOP = false>
 __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, const KH &kh, int k, uint32_t m,
                                                uint32_t w0, const R (&z)[D], const R (&uk)[DU], R (&x)[D],
-                                               LW &lw) {
+                                               LW &lw, SlotScratch<R, D> *sc = nullptr) {
   using M = Ar<R>;
   constexpr bool LOG = !std::is_same<LW, NoLog>::value;
+  if constexpr (COOP) {   // every lane of the warp is here
+    const bool one = has_jump(kp, w0) && one_jump(kp, w0);
+    const unsigned om = __ballot_sync(0xffffffffu, one);
+    if (om) {
+      R th = R(0), xih[D], z1[D];
+      coop_slot0_draws(kp, *sc, k, m, om, th, xih, z1);
+      if (one) {
+        one_jump_inline(kp, k, th, xih, z, z1, uk, x, lw);
+        return 1;
+      }
+    }
+  }
   if (!has_jump(kp, w0)) {
     R f[D];
     drift(kh, x, uk, f);
@@ -394,7 +456,7 @@ __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, cons
     }
     return 1;
   }
-  if (INLINE_JUMP && one_jump(kp, w0)) {
+  if (!COOP && INLINE_JUMP && one_jump(kp, w0)) {
     R xih[D], z1[D];
     const R th = slot0_draws<RK>(kp, k, m, xih, z1);
     one_jump_inline(kp, k, th, xih, z, z1, uk, x, lw);
@@ -431,10 +493,10 @@ __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, cons
 // the post-jump states of the step are recorded.  zo (optional, stride zs) receives the
 // step's main-stream normals Z_{k,0}.
 template <typename R, int D, int DU, typename LW, bool ZOUT = false, bool INLINE_JUMP = true,
-          typename KH = KParams<R, D, DU>, bool RK = false>
+          typename KH = KParams<R, D, DU>, bool RK = false, bool COOP = false>
 __device__ __forceinline__ int forward_step_h(const KParams<R, D, DU> &kp, const KH &kh, int k, uint32_t m,
                                               const R *__restrict__ u, R (&x)[D], LW &lw,
-                                              R *zo = nullptr, int zs = 0) {
+                                              R *zo = nullptr, int zs = 0, SlotScratch<R, D> *sc = nullptr) {
   R z[D];
   const uint32_t w0 = main_draws<RK>(kp, k, m, z);
   if constexpr (ZOUT) {
@@ -444,14 +506,15 @@ __device__ __forceinline__ int forward_step_h(const KParams<R, D, DU> &kp, const
   R uk[DU];
 #pragma unroll
   for (int l = 0; l < DU; ++l) uk[l] = __ldg(u + (size_t)k * DU + l);
-  return step_from_draws<R, D, DU, LW, INLINE_JUMP, KH, RK>(kp, kh, k, m, w0, z, uk, x, lw);
+  return step_from_draws<R, D, DU, LW, INLINE_JUMP, KH, RK, COOP>(kp, kh, k, m, w0, z, uk, x, lw, sc);
 }
 
-template <typename R, int D, int DU, typename LW, bool ZOUT = false, bool INLINE_JUMP = true>
+template <typename R, int D, int DU, typename LW, bool ZOUT = false, bool INLINE_JUMP = true, bool COOP = false>
 __device__ __forceinline__ int forward_step(const KParams<R, D, DU> &kp, int k, uint32_t m,
                                             const R *__restrict__ u, R (&x)[D], LW &lw,
-                                            R *zo = nullptr, int zs = 0) {
-  return forward_step_h<R, D, DU, LW, ZOUT, INLINE_JUMP>(kp, kp, k, m, u, x, lw, zo, zs);
+                                            R *zo = nullptr, int zs = 0, SlotScratch<R, D> *sc = nullptr) {
+  return forward_step_h<R, D, DU, LW, ZOUT, INLINE_JUMP, KParams<R, D, DU>, false, COOP>(kp, kp, k, m, u, x, lw, zo,
+                                                                                        zs, sc);
 }
 
 // Step k of two controls u, u2 on the same random data (the pair of Armijo trials of one
@@ -594,9 +657,34 @@ inline int fwd_chunk_len(double lamdt, int most) {
 // (double precision, M = 2^15: store sweep 1.17 -> 1.17, 1.30 -> 1.28, 1.68 -> 1.49, 2.68 ->
 // 2.17, 4.32 -> 4.14 ms up to 0.2.)  Between 0.004 and 0.007 the forms are within 3%.
 constexpr double FWD_CHUNK_RATE = 0.006;
+// What a launch runs: a sweep without stored states, the single store sweep, the replay of the
+// recompute adjoint.
+enum SweepKind { SWEEP_PLAIN, SWEEP_STORE, SWEEP_REPLAY };
+
+// d > 2: whether a one-jump step's slot draws are the whole warp's (coop_slot0_draws).  A lane
+// alone draws with its warp waiting; the warp-wide form costs the steps without jumps a
+// ballot and registers, and takes the jump lanes one after another, so it pays between a
+// lowest and a highest jump rate per step.  One launch, N_t = 160, one lane -> warp, in ms:
+//   lambda dt                        0              0.002          0.01           0.05
+//   FP32 d = 8  M = 200,003  cost    0.65 -> 0.67   0.75 -> 0.71   1.04 -> 0.87   2.45 -> 1.78
+//                            store   0.71 -> 0.78   0.80 -> 0.83   1.13 -> 1.01   2.51 -> 2.22
+//                            replay  1.04 -> 1.08   1.37 -> 1.20   2.81 -> 2.00   6.24 -> 5.08
+//   FP32 d = 4               cost    0.34 -> 0.37   0.38 -> 0.40   0.50 -> 0.50   0.89 -> 0.94
+//                            replay  0.57 -> 0.57   0.63 -> 0.61   0.81 -> 0.76   1.76 -> 1.57
+//   FP64 d = 8  M = 16,000   store   1.86 -> 1.86   2.20 -> 2.00   3.08 -> 2.50   5.63 -> 4.20
+//   FP64 d = 4               store   0.87 -> 0.88   1.02 -> 0.94   1.44 -> 1.20   2.53 -> 2.15
+// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)
 template <typename R, int D>
-inline bool fwd_chunks(double lamdt, bool single_store) {
-  return fwd_chunked<D>() && (sizeof(R) == 8 || single_store || lamdt > FWD_CHUNK_RATE);
+inline bool coop_slots(double lamdt, SweepKind kind) {
+  if (sizeof(R) == 8) return lamdt > 0.0005 && lamdt <= 0.1;
+  if (D == 8) return lamdt > (kind == SWEEP_STORE ? 0.005 : 0.0015) && lamdt <= 0.08;
+  return kind == SWEEP_REPLAY ? lamdt > 0.003 && lamdt <= 0.08 : lamdt > 0.01 && lamdt <= 0.03;
+}
+
+template <typename R, int D>
+inline bool fwd_chunks(double lamdt, SweepKind kind) {
+  if (!fwd_chunked<D>()) return coop_slots<R, D>(lamdt, kind);
+  return sizeof(R) == 8 || kind == SWEEP_STORE || lamdt > FWD_CHUNK_RATE;
 }
 
 // Bits of a chunk, bit i for its step i: jumps; two or more; the jumps have records (in
@@ -1314,13 +1402,14 @@ __device__ __forceinline__ void one_jump_pre(const KParams<R, D, DU> &kp, int k,
 // block_sum_to_double does in the one-path-per-thread launch.
 // RK: kp is the launch's __grid_constant__ parameter, whose Philox round keys the draws
 // take as constant operands (fwd_kernel); the batched sweeps' kp lies in a table.
-template <typename R, int D, int DU, int MODE, bool PAIR = false, bool PRE = false, bool RK = false>
+template <typename R, int D, int DU, int MODE, bool PAIR = false, bool PRE = false, bool RK = false,
+          bool COOP = false>
 __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bid, const R *__restrict__ u,
                                          const R *__restrict__ xd, double *__restrict__ partC, R *__restrict__ traj,
                                          uint32_t *__restrict__ flags, R *__restrict__ ckpt, R *__restrict__ pcost,
                                          const JLog<R, D> &jl, int *__restrict__ jcnt, int64_t mloc,
                                          const PairOut<R, D> &p2, const PreDraws<R, D> &pd, Pair<R> *red,
-                                         PreRing<R, D, DU> *ring = nullptr) {
+                                         PreRing<R, D, DU> *ring = nullptr, SlotScratch<R, D> *slots = nullptr) {
   if (PRE && threadIdx.x >= SPREAD_LANES) return;   // no warp-wide operation follows in this mode
   const int64_t lm = PRE ? bid * SPREAD_LANES + threadIdx.x : bid * TPB + threadIdx.x;
   const bool active = lm < mloc;
@@ -1411,7 +1500,7 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
       const uint32_t w0 = main_draws<RK>(kp, k, m, z);
       nj = forward_step2<R, D, DU, LW, KH, RK>(kp, kh, k, m, w0, z, u, x, lw, p2.u, x2, lw2);
     } else {
-      nj = forward_step_h<R, D, DU, LW, false, true, KH, RK>(kp, kh, k, m, u, x, lw);
+      nj = forward_step_h<R, D, DU, LW, false, true, KH, RK, COOP>(kp, kh, k, m, u, x, lw, nullptr, 0, slots);
     }
     if (nj) fw |= 1u << (k & 31);
     if constexpr (PRE)
@@ -1682,6 +1771,10 @@ fwd_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u
     __shared__ PreRing<R, D, DU> ring;
     fwd_body<R, D, DU, MODE, PAIR, PRE, RK>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt, mloc,
                                             p2, pd, red, &ring);
+  } else if constexpr (CHUNK && D > 2) {
+    __shared__ SlotScratch<R, D> slots[TPB / 32];
+    fwd_body<R, D, DU, MODE, PAIR, PRE, RK, true>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt,
+                                                  mloc, p2, pd, red, nullptr, &slots[threadIdx.x >> 5]);
   } else if constexpr (CHUNK) {
     __shared__ FwdChunkSmem<R, D, PAIR> sm;
     fwd_chunk_body<R, D, DU, MODE, PAIR, true, 4>(kp, blockIdx.x, u, xd, partC, traj, flags, ckpt, pcost, jl, jcnt,
@@ -2022,6 +2115,11 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
   GradRows<R, DU, NR> rows;
   rows.init(sy + (size_t)JS * D * TPB);
   R(*const srec)[TPB] = reinterpret_cast<R(*)[TPB]>(sy + (size_t)JS * D * TPB + grad_rows_bytes<R, DU, 8>() / sizeof(R));
+  SlotScratch<R, D> *slots = nullptr;   // d > 2: the replay's warp-wide slot draws
+  if constexpr (D > 2 && RCH) {
+    __shared__ SlotScratch<R, D> slot_sm[TPB / 32];
+    slots = &slot_sm[threadIdx.x >> 5];
+  }
   __shared__ Pair<R> red1[TPB / 32];
   const int64_t npart = kp.npart;
   const int64_t lm = (int64_t)blockIdx.x * TPB + threadIdx.x;
@@ -2053,7 +2151,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
       lw.L = sl;
       lw.idx = tid;
     }
-    if constexpr (RCH) {
+    if constexpr (RCH && D <= 2) {
       // chunks of the replay: the step's normals wait where its state will lie
 #pragma unroll 1
       for (int c0 = 0; c0 < len; c0 += kp.chunk) {
@@ -2086,8 +2184,8 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
       for (int i = 0; i < len; ++i) {
   #pragma unroll
         for (int c = 0; c < D; ++c) sbuf[(i * D + c) * TPB + tid] = x[c];
-        if (forward_step<R, D, DU, LWR, ZBUF, !THETA>(kp, k0 + i, m, u, x, lw, zbuf + (size_t)i * D * TPB + tid,
-                                                      TPB))
+        if (forward_step<R, D, DU, LWR, ZBUF, !THETA, (D > 2 && RCH)>(
+                kp, k0 + i, m, u, x, lw, zbuf + (size_t)i * D * TPB + tid, TPB, slots))
           jm |= 1ull << i;
       }
     }
@@ -2118,7 +2216,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
         for (int j = CH - 1; j >= 0; --j) {
           const int i = i0 + j;
           R g[DU], xk[D], xdk[D];
-          seg_state<R, D, RCH>(sbuf, i, xk);
+          seg_state<R, D, (RCH && D <= 2)>(sbuf, i, xk);
           load_row<R, D>(xdc + j * D, xdk);
           backward_logged(kp, xk, mu, g, lr, (jwm >> j) & 1u, (jm >> i) & 1u);
           cost_gradient(kp, xk, xdk, mu);
@@ -2134,7 +2232,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
           for (int l = 0; l < DU; ++l) g[l] = R(0);
           if (i < len) {
             R xk[D];
-            seg_state<R, D, RCH>(sbuf, i, xk);
+            seg_state<R, D, (RCH && D <= 2)>(sbuf, i, xk);
             const bool jumped = (jm >> i) & 1u;
             if constexpr (THETA) {
               backward_step<R, D, DU, true, LogReader<R, D>, ZBUF>(kp, kp, k, m, jumped, xk, u, xd, mu, g, th, lr0,
@@ -2402,7 +2500,7 @@ __device__ __forceinline__ void adj_theta_body(const KParams<R, D, DU> &kp, cons
   finish_theta<R, D, DU, true>(kp, th, active, partT, red1, blockIdx.x);
 }
 
-// CHUNK: the replay in chunks (u-gradient, d <= 2), or the kept jump draws (parameter
+// CHUNK: the replay in chunks (u-gradient, d <= 2) or with warp-wide slot draws (d > 2), or the kept jump draws (parameter
 // gradients); the host's rule (op_adj).
 template <typename R, int D, int DU, bool THETA, bool CHUNK = false>
 __global__ void __launch_bounds__(TPB)
@@ -2445,7 +2543,7 @@ auto recompute_form(bool theta, bool chunk) {
       k = chunk ? &adj_recompute_kernel<R, D, DU, true, true> : &adj_recompute_kernel<R, D, DU, true>;
     else
       k = &adj_recompute_kernel<R, D, DU, true>;
-  } else if constexpr (fwd_chunked<D>()) {
+  } else {
     if (chunk) k = &adj_recompute_kernel<R, D, DU, false, true>;
   }
   return k;
@@ -2558,11 +2656,11 @@ unsigned long long draws_key(const KParams<R, D, DU> &kp, int64_t mloc) {
   return h | 1ull;
 }
 
-// The sweep's kernel: in chunks or step by step.
+// The sweep's kernel: in chunks (d <= 2) or with warp-wide slot draws (d > 2), or step by step.
 template <typename R, int D, int DU, int MODE, bool PAIR = false>
 auto fwd_form(bool chunk) {
   auto k = &fwd_kernel<R, D, DU, MODE, PAIR>;
-  if constexpr (fwd_chunked<D>()) {
+  if constexpr (D <= 8 && !(PAIR && D > 2)) {
     if (chunk) k = &fwd_kernel<R, D, DU, MODE, PAIR, false, true>;
   }
   return k;
@@ -2624,7 +2722,8 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
       return cudaGetLastError();
     }
   }
-  const bool chunk = fwd_chunks<R, D>(p->desc.lambda * p->desc.T / (double)p->desc.Nt, mode == FWD_STORE);
+  const bool chunk = fwd_chunks<R, D>(p->desc.lambda * p->desc.T / (double)p->desc.Nt,
+                                       mode == FWD_STORE ? SWEEP_STORE : SWEEP_PLAIN);
   switch (mode) {
     case FWD_COST:
       fwd_form<R, D, DU, FWD_COST>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr, nullptr, pc, jl,
@@ -2729,7 +2828,7 @@ cudaError_t op_adj(const jd_problem *p, int variant, bool theta, int64_t m_begin
   } else {
     const R *ck = static_cast<const R *>(b.ckpt);
     const double lamdt = p->desc.lambda * p->desc.T / (double)p->desc.Nt;
-    const bool chunk = theta ? lamdt <= THETA_KEEP_RATE : fwd_chunks<R, D>(lamdt, false);
+    const bool chunk = theta ? lamdt <= THETA_KEEP_RATE : fwd_chunks<R, D>(lamdt, SWEEP_REPLAY);
     const size_t smem = recompute_smem_form<R, D, DU>(theta, chunk, kp.S);
     const auto k = recompute_form<R, D, DU>(theta, chunk);
     err = ensure_dyn_smem((const void *)k, smem);

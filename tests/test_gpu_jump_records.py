@@ -76,3 +76,28 @@ def test_chunked_pairs_equal_single_trials(prec, lamdt):
             out.append((v, hist, r["evals"]))
     for v, hist, evals in out[1:]:
         assert np.array_equal(v, out[0][0]) and np.array_equal(hist, out[0][1]) and evals == out[0][2]
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("d", [3, 4, 8])
+def test_warp_wide_slot_draws_equal_single_lanes(d, prec):
+    """For d > 2 the rate per step decides whether a jump step's draws are the warp's or the
+    lane's, and the store and replay sweeps have different limits: across them the plans agree
+    bit for bit, and the costs of the same paths (sums over the path) with the oracle."""
+    import oracle
+    for lamdt in (0.0002, 0.002, 0.007, 0.04, 0.09, 0.5):
+        Nt, M = 37, 1001
+        p = workloads.linear_family(d, M, Nt, lam=lamdt * Nt, seed=12)
+        u = workloads.random_control(p, seed=3, scale=0.6)
+        out = []
+        for mode in ("stored", "recompute"):
+            with JdProblem(p, prec=prec, mode=mode) as jp:
+                J, g, _ = jp.gradient(u)
+                X, _, c = jp.sample_paths(u, 0, M, lam=False)
+            out.append((J, g, X, c))
+        for a, b in zip(*out):
+            assert np.array_equal(a, b)
+        tol = 1e-5 if prec == "fp32" else 1e-12
+        for m in range(0, M, 97):
+            r = oracle.path(p, u, m)
+            assert abs(out[0][3][m] - r["cost"]) <= tol * abs(r["cost"])
