@@ -142,13 +142,19 @@ constexpr int RING_MAX = 2048;   // 8 blocks of 256 lanes: the largest portable 
 // step sit on that chain) takes its main-stream draws in one parallel kernel first, when
 // their buffers stay small.  Its sweeps then run few lanes per warp (SPREAD_LANES), which
 // costs them instruction issue as the paths grow: the limits are where three projected-
-// gradient iterations take as long with the chunked sweeps (N_t = 200, lambda dt = 0.02,
-// pre-drawn / chunked in us):
-//   FP32 d = 1  M = 4000  805 / 897    8000  903 / 939    16000  1180 / 955   32000  2144 / 1062
-//   FP32 d = 2            817 / 914          946 / 972           1394 / 1009
-//   FP64 d = 1           2246 / 3873        3585 / 3900          6239 / 4002
-//   FP64 d = 2           4106 / 5453        6592 / 5490
-inline int64_t pre_max_paths(int D, size_t es) { return es == 4 ? 152 * 64 : D == 1 ? 152 * 48 : 152 * 32; }
+// gradient iterations take as long with the chunked sweeps (N_t = 200, pre-drawn / chunked
+// in us, by lambda dt):
+//                          0.002         0.02          0.1
+//   FP32 d = 1  M = 8000   746 / 597     902 / 854     1489 / 1565
+//               M = 10000  820 / 587     999 / 848     1627 / 1562
+//   FP64 d = 1  M = 7500   2863 / 2839   3464 / 3856   5909 / 6436
+//               M = 9000   3337 / 2845   3982 / 3851   7063 / 6409
+//   FP64 d = 2  M = 6000   4358 / 4022   5200 / 5394   7924 / 8960
+//               M = 7500   5387 / 4014   6401 / 5407   9792 / 8967
+inline int64_t pre_max_paths(int D, size_t es, double lamdt) {
+  if (es == 4) return lamdt > 0.05 ? 152 * 64 : 152 * 40;
+  return D == 1 ? 152 * 56 : 152 * 40;
+}
 constexpr size_t PRE_MAX_BYTES = (size_t)128 << 20;
 // pre_z holds the normals, the slot-0 draws and then the paths' cost pairs of the sweeps
 // (2 controls x M pairs of 2 values)
@@ -159,9 +165,9 @@ inline size_t pre_bytes(int Nt, int D, int64_t M, size_t es) {
   // words; normals, slot-0 draws and cost pairs; the key of the draws held
   return (size_t)Nt * (size_t)M * 4 + pre_z_values(Nt, D, M) * es + sizeof(unsigned long long);
 }
-inline bool pre_pass(int d, int Nt, int64_t M, size_t es) {
+inline bool pre_pass(int d, int Nt, int64_t M, size_t es, double lamdt) {
   const int D = d <= 1 ? 1 : 2;
-  return d <= 2 && M <= pre_max_paths(D, es) && pre_bytes(Nt, D, M, es) <= PRE_MAX_BYTES;
+  return d <= 2 && M <= pre_max_paths(D, es, lamdt) && pre_bytes(Nt, D, M, es) <= PRE_MAX_BYTES;
 }
 
 struct FbBufs {
