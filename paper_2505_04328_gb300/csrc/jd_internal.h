@@ -8,6 +8,7 @@
 #include <vector>
 
 #include "jd.h"
+#include "jd_rules.h"
 
 namespace jd {
 
@@ -165,7 +166,10 @@ inline size_t pre_bytes(int Nt, int D, int64_t M, size_t es) {
   // words; normals, slot-0 draws and cost pairs; the key of the draws held
   return (size_t)Nt * (size_t)M * 4 + pre_z_values(Nt, D, M) * es + sizeof(unsigned long long);
 }
-inline bool pre_pass(int d, int Nt, int64_t M, size_t es, double lamdt) {
+inline bool pre_pass(const jd_problem_desc &q, size_t es) {
+  const int d = q.d, Nt = q.Nt;
+  const int64_t M = q.M;
+  const double lamdt = jump_rate(q.jump_law, q.lambda, q.T, Nt);
   const int D = d <= 1 ? 1 : 2;
   return d <= 2 && M <= pre_max_paths(D, es, lamdt) && pre_bytes(Nt, D, M, es) <= PRE_MAX_BYTES;
 }

@@ -635,58 +635,6 @@ struct FwdChunk {
   // the noise scales sigma sqrt(delta) of its two sub-steps
   static constexpr int TH = 0, XJ = 1, Z1 = 1 + D, A0 = 1 + 2 * D, A1 = 1 + 3 * D, W = 1 + 4 * D;
 };
-// Chunk length: the records hold a lane's jumps of a chunk but in rare chunks, and a pass of
-// slot draws serves many lanes.
-inline int fwd_chunk_len(double lamdt, int most) {
-  const int n = lamdt <= 0.015 ? 16 : lamdt <= 0.03 ? 8 : 4;
-  return n < most ? n : most;
-}
-
-// Whether a sweep takes its steps in chunks, by the jump rate per step.  The store sweep and
-// every FP64 sweep gain or tie at any rate; the other FP32 sweeps pay about 6% for the
-// chunks' passes without jumps and gain from about lambda dt = 0.005 on.  One launch at M =
-// 2^20, N_t = 160, d = 2 FP32, step by step -> in chunks, in ms:
-//   lambda dt          0            0.002         0.01          0.05          0.2           0.4
-//   cost          0.91 -> 0.97  1.01 -> 1.06  1.32 -> 1.23  2.33 -> 1.94  5.88 -> 3.27  9.96 -> 7.08
-//   store         1.11 -> 1.04  1.21 -> 1.15  1.56 -> 1.38  2.66 -> 2.24  6.38 -> 3.83  10.5 -> 8.48
-//   checkpoints   0.94 -> 0.99  1.02 -> 1.09  1.32 -> 1.25  2.30 -> 1.97  5.97 -> 3.34  10.1 -> 7.55
-//   store, pair   1.25 -> 1.22  1.38 -> 1.39  1.82 -> 1.79  4.16 -> 3.03  12.9 -> 6.65  21.9 -> 15.7
-//   ckpt., pair   1.11 -> 1.15  1.21 -> 1.27  1.59 -> 1.51  3.16 -> 2.44  10.1 -> 4.69  18.4 -> 11.9
-//   recompute     1.26 -> 1.35  1.39 -> 1.47  1.80 -> 1.70  3.18 -> 2.75  12.1 -> 12.1  23.7 -> 22.1
-//   adjoint (replay)
-// (double precision, M = 2^15: store sweep 1.17 -> 1.17, 1.30 -> 1.28, 1.68 -> 1.49, 2.68 ->
-// 2.17, 4.32 -> 4.14 ms up to 0.2.)  Between 0.004 and 0.007 the forms are within 3%.
-constexpr double FWD_CHUNK_RATE = 0.006;
-// What a launch runs: a sweep without stored states, the single store sweep, the replay of the
-// recompute adjoint.
-enum SweepKind { SWEEP_PLAIN, SWEEP_STORE, SWEEP_REPLAY };
-
-// d > 2: whether a one-jump step's slot draws are the whole warp's (coop_slot0_draws).  A lane
-// alone draws with its warp waiting; the warp-wide form costs the steps without jumps a
-// ballot and registers, and takes the jump lanes one after another, so it pays between a
-// lowest and a highest jump rate per step.  One launch, N_t = 160, one lane -> warp, in ms:
-//   lambda dt                        0              0.002          0.01           0.05
-//   FP32 d = 8  M = 200,003  cost    0.65 -> 0.67   0.75 -> 0.71   1.04 -> 0.87   2.45 -> 1.78
-//                            store   0.71 -> 0.78   0.80 -> 0.83   1.13 -> 1.01   2.51 -> 2.22
-//                            replay  1.04 -> 1.08   1.37 -> 1.20   2.81 -> 2.00   6.24 -> 5.08
-//   FP32 d = 4               cost    0.34 -> 0.37   0.38 -> 0.40   0.50 -> 0.50   0.89 -> 0.94
-//                            replay  0.57 -> 0.57   0.63 -> 0.61   0.81 -> 0.76   1.76 -> 1.57
-//   FP64 d = 8  M = 16,000   store   1.86 -> 1.86   2.20 -> 2.00   3.08 -> 2.50   5.63 -> 4.20
-//   FP64 d = 4               store   0.87 -> 0.88   1.02 -> 0.94   1.44 -> 1.20   2.53 -> 2.15
-// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)
-template <typename R, int D>
-inline bool coop_slots(double lamdt, SweepKind kind) {
-  if (sizeof(R) == 8) return lamdt > 0.0005 && lamdt <= 0.1;
-  if (D == 8) return lamdt > (kind == SWEEP_STORE ? 0.005 : 0.0015) && lamdt <= 0.08;
-  return kind == SWEEP_REPLAY ? lamdt > 0.003 && lamdt <= 0.08 : lamdt > 0.01 && lamdt <= 0.03;
-}
-
-template <typename R, int D>
-inline bool fwd_chunks(double lamdt, SweepKind kind) {
-  if (!fwd_chunked<D>()) return coop_slots<R, D>(lamdt, kind);
-  return sizeof(R) == 8 || kind == SWEEP_STORE || lamdt > FWD_CHUNK_RATE;
-}
-
 // Bits of a chunk, bit i for its step i: jumps; two or more; the jumps have records (in
 // record order); some lane of the warp jumps (warp-uniform: the steps pass runs a step in
 // which no lane jumps without a test per lane).
@@ -2549,12 +2497,6 @@ auto recompute_form(bool theta, bool chunk) {
   return k;
 }
 
-// Parameter gradients: the jump draws are kept up to this jump rate per step; beyond it a
-// segment's jumps outgrow the records and most steps have several (M = 2^19, N_t = 160, d = 2
-// FP32, regenerated -> kept: 0.80 -> 0.86 ms without jumps, 1.36 -> 0.94 at 0.002, 3.29 ->
-// 1.16 at 0.01, 7.82 -> 4.16 at 0.05, 10.9 -> 9.8 at 0.1, 16.0 -> 20.0 at 0.2).
-constexpr double THETA_KEEP_RATE = 0.12;
-
 // ---------------------------------------------------------------------------
 // Host-side launch ops for one (precision, D, DU)
 // ---------------------------------------------------------------------------
@@ -2625,7 +2567,8 @@ void make_kparams(const jd_problem *p, int64_t m_begin, int64_t mloc, KParams<R,
   kp.jumps_on = q.jump_law != JD_JUMP_NONE && q.lambda > 0.0;
   kp.has_dA = !p->dA.empty();
   kp.chunk = 4;
-  if constexpr (fwd_chunked<D>()) kp.chunk = fwd_chunk_len(q.lambda * dt, FwdChunk<R, D>::CH);
+  if constexpr (fwd_chunked<D>())
+    kp.chunk = fwd_chunk_len(jump_rate(q.jump_law, q.lambda, q.T, q.Nt), FwdChunk<R, D>::CH);
   kp.S = p->S;   // checkpoint spacing of the recompute plan (a power of two, 16 .. 64)
   kp.nblk = (int)ceil_div(mloc, TPB);
   kp.m_begin = q.m_offset + m_begin;   // global path index (a shard starts at m_offset)
@@ -2722,8 +2665,7 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
       return cudaGetLastError();
     }
   }
-  const bool chunk = fwd_chunks<R, D>(p->desc.lambda * p->desc.T / (double)p->desc.Nt,
-                                       mode == FWD_STORE ? SWEEP_STORE : SWEEP_PLAIN);
+  const bool chunk = fwd_chunks(form_key(D, sizeof(R) == 8, p->desc), mode == FWD_STORE ? SWEEP_STORE : SWEEP_PLAIN);
   switch (mode) {
     case FWD_COST:
       fwd_form<R, D, DU, FWD_COST>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr, nullptr, pc, jl,
@@ -2827,8 +2769,8 @@ cudaError_t op_adj(const jd_problem *p, int variant, bool theta, int64_t m_begin
     }
   } else {
     const R *ck = static_cast<const R *>(b.ckpt);
-    const double lamdt = p->desc.lambda * p->desc.T / (double)p->desc.Nt;
-    const bool chunk = theta ? lamdt <= THETA_KEEP_RATE : fwd_chunks<R, D>(lamdt, SWEEP_REPLAY);
+    const FormKey form = form_key(D, sizeof(R) == 8, p->desc);
+    const bool chunk = theta ? theta_keeps(form) : fwd_chunks(form, SWEEP_REPLAY);
     const size_t smem = recompute_smem_form<R, D, DU>(theta, chunk, kp.S);
     const auto k = recompute_form<R, D, DU>(theta, chunk);
     err = ensure_dyn_smem((const void *)k, smem);

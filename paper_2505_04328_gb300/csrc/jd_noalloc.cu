@@ -111,7 +111,7 @@ static void noalloc_kparams(const jd_problem_desc &q, KParams<R, D, DU> &kp) {
   kp.jumps_on = q.jump_law != JD_JUMP_NONE && q.lambda > 0.0;
   kp.has_dA = 0;
   kp.S = seg_len<D>();
-  kp.chunk = fwd_chunk_len(q.lambda * dt, FwdChunk<R, D>::CH);
+  kp.chunk = fwd_chunk_len(jump_rate(q.jump_law, q.lambda, q.T, q.Nt), FwdChunk<R, D>::CH);
   kp.nblk = (int)ceil_div(q.M, TPB);
   kp.m_begin = q.m_offset;   // global index of the first path
   kp.npart = kp.nblk * (int64_t)(TPB / 32);
@@ -141,7 +141,7 @@ static jd_status noalloc_run(const jd_problem_desc &q, unsigned char *scratch, c
   KParams<R, D, 1> kp;
   noalloc_kparams<R, D, 1>(q, kp);
   const JLog<R, D> nolog{nullptr, nullptr, M, 0};
-  const auto k = fwd_form<R, D, 1, FWD_COST>(fwd_chunks<R, D>(q.lambda * (q.T / (double)Nt), SWEEP_PLAIN));
+  const auto k = fwd_form<R, D, 1, FWD_COST>(fwd_chunks(form_key(D, sizeof(R) == 8, q), SWEEP_PLAIN));
   k<<<(unsigned)nblk, TPB, 0, s>>>(kp, uk, xdk, partC, nullptr, nullptr, nullptr, nullptr, nolog, nullptr, M,
                                    PairOut<R, D>{}, PreDraws<R, D>{});
   noalloc_finalize_kernel<<<1, 256, 0, s>>>(partC, nblk, u, Nt, 0.5 * q.nu * (q.T / Nt), 1.0 / (double)M, J);

@@ -1,0 +1,83 @@
+"""The host rules that choose a sweep's form (jd_rules.h), compiled here for this host."""
+import ctypes
+import os
+import subprocess
+
+import pytest
+
+from paper_2505_04328_gb300 import _build
+
+NONE, NORMAL, UNIFORM, KS = range(4)
+PLAIN, STORE, REPLAY = range(3)
+
+SRC = r"""
+#include "jd_rules.h"
+using namespace jd;
+static jd_problem_desc desc(int d, int law, double rate) {
+  jd_problem_desc q{};
+  q.d = d;
+  q.T = 2.0;
+  q.Nt = 64;
+  q.lambda = rate * 32.0;
+  q.jump_law = (jd_jump_law)law;
+  return q;
+}
+static FormKey key(int d, int f64, int law, double rate) {
+  return form_key(d <= 2 ? d : d <= 4 ? 4 : 8, f64 != 0, desc(d, law, rate));
+}
+extern "C" {
+double rate_of(int law, double lambda, double T, int Nt) { return jump_rate((jd_jump_law)law, lambda, T, Nt); }
+int chunk_len(int d, int law, double rate, int most) { return fwd_chunk_len(key(d, 0, law, rate).rate, most); }
+int chunks(int d, int f64, int law, double rate, int kind) {
+  return fwd_chunks(key(d, f64, law, rate), (SweepKind)kind);
+}
+int keeps(int d, int f64, int law, double rate) { return theta_keeps(key(d, f64, law, rate)); }
+}
+"""
+
+
+@pytest.fixture(scope="module")
+def rules(tmp_path_factory):
+    d = tmp_path_factory.mktemp("rules")
+    src, lib = os.path.join(d, "rules.cpp"), os.path.join(d, "rules.so")
+    with open(src, "w") as f:
+        f.write(SRC)
+    r = subprocess.run(["g++", "-std=c++17", "-Wall", "-Werror", "-Wno-unused-function", "-shared", "-fPIC",
+                        "-I", _build.CSRC, "-I", _build.INCLUDE, src, "-o", lib], capture_output=True, text=True)
+    assert r.returncode == 0, r.stderr[-3000:]
+    so = ctypes.CDLL(lib)
+    so.rate_of.restype = ctypes.c_double
+
+    class Rules:
+        @staticmethod
+        def rate(law, lam, T, Nt):
+            return so.rate_of(law, ctypes.c_double(lam), ctypes.c_double(T), Nt)
+
+        @staticmethod
+        def chunk_len(d, law, rate, most=16):
+            return so.chunk_len(d, law, ctypes.c_double(rate), most)
+
+        @staticmethod
+        def chunks(d, f64, law, rate, kind):
+            return bool(so.chunks(d, int(f64), law, ctypes.c_double(rate), kind))
+
+        @staticmethod
+        def keeps(d, f64, law, rate):
+            return bool(so.keeps(d, int(f64), law, ctypes.c_double(rate)))
+
+    return Rules
+
+
+@pytest.mark.parametrize("f64", [False, True])
+@pytest.mark.parametrize("d", [1, 2, 4, 8])
+def test_a_problem_without_a_jump_law_has_no_rate(rules, d, f64):
+    """Its intensity may be set: every form is then the one of rate 0 (FP32 d = 8 store sweep
+    without jumps 0.473 -> 0.508 ms in the form for jumps)."""
+    assert rules.rate(NONE, 5.0, 2.0, 100) == 0.0 and rules.rate(NORMAL, 5.0, 2.0, 100) == 0.1
+    for rate in (0.002, 0.01, 0.05, 0.3):
+        assert rules.chunk_len(d, NONE, rate) == 16
+        for kind in (PLAIN, STORE, REPLAY):
+            assert rules.chunks(d, f64, NONE, rate, kind) == rules.chunks(d, f64, NORMAL, 0.0, kind)
+        assert rules.keeps(d, f64, NONE, rate) == rules.keeps(d, f64, NORMAL, 0.0)
+    if d > 2:
+        assert not any(rules.chunks(d, f64, NONE, 0.01, kind) for kind in (PLAIN, STORE, REPLAY))
