@@ -16,10 +16,14 @@ inline double jump_rate(jd_jump_law law, double lambda, double T, int Nt) {
 struct FormKey {
   int D;
   bool f64;
-  double rate;   // jump_rate
+  bool one_jump;   // steps with one jump take the short path (one_jump of the kernels): the
+                   // slot's words lie as compiled for D, and the law is additive for d > 2
+  double rate;     // jump_rate
 };
 inline FormKey form_key(int D, bool f64, const jd_problem_desc &q) {
-  return FormKey{D, f64, jump_rate(q.jump_law, q.lambda, q.T, q.Nt)};
+  const bool packed = (q.d + 1) / 2 == (D + 1) / 2;
+  return FormKey{D, f64, packed && (D <= 2 || q.jump_law != JD_JUMP_KS),
+                 jump_rate(q.jump_law, q.lambda, q.T, q.Nt)};
 }
 
 // Chunk length: the records hold a lane's jumps of a chunk but in rare chunks, and a pass of
@@ -60,8 +64,11 @@ enum SweepKind { SWEEP_PLAIN, SWEEP_STORE, SWEEP_REPLAY };
 //                            replay  0.57 -> 0.57   0.63 -> 0.61   0.81 -> 0.76   1.76 -> 1.57
 //   FP64 d = 8  M = 16,000   store   1.86 -> 1.86   2.20 -> 2.00   3.08 -> 2.50   5.63 -> 4.20
 //   FP64 d = 4               store   0.87 -> 0.88   1.02 -> 0.94   1.44 -> 1.20   2.53 -> 2.15
-// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)
+// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)  Where no
+// step takes the one-jump path the form only costs: Keilson-Storer d = 8, FP32, M = 2^17, store
+// sweep 1.17 -> 1.33 ms at 0.01, 1.52 -> 1.83 at 0.02, cost 1.07 -> 1.17 and 1.47 -> 1.63.
 inline bool coop_slots(const FormKey &f, SweepKind kind) {
+  if (!f.one_jump) return false;
   if (f.f64) return f.rate > 0.0005 && f.rate <= 0.1;
   if (f.D == 8) return f.rate > (kind == SWEEP_STORE ? 0.005 : 0.0015) && f.rate <= 0.08;
   return kind == SWEEP_REPLAY ? f.rate > 0.003 && f.rate <= 0.08 : f.rate > 0.01 && f.rate <= 0.03;

@@ -81,3 +81,17 @@ def test_a_problem_without_a_jump_law_has_no_rate(rules, d, f64):
         assert rules.keeps(d, f64, NONE, rate) == rules.keeps(d, f64, NORMAL, 0.0)
     if d > 2:
         assert not any(rules.chunks(d, f64, NONE, 0.01, kind) for kind in (PLAIN, STORE, REPLAY))
+
+
+@pytest.mark.parametrize("f64", [False, True])
+def test_warp_wide_draws_need_a_one_jump_path(rules, f64):
+    """Keilson-Storer steps of d > 2, and dimensions whose slot words are packed for fewer
+    pairs than compiled (d = 5, 6 in the kernels of d = 8), have no one-jump path: the
+    warp-wide form would cost and give nothing (KS d = 8, FP32, 0.02: store 1.52 -> 1.83 ms)."""
+    rates = (0.002, 0.006, 0.012, 0.02, 0.05, 0.08)
+    kinds = (PLAIN, STORE, REPLAY)
+    for d in (3, 4, 7, 8):
+        assert not any(rules.chunks(d, f64, KS, r, k) for r in rates for k in kinds)
+        assert any(rules.chunks(d, f64, NORMAL, r, k) for r in rates for k in kinds)
+    for d in (5, 6):
+        assert not any(rules.chunks(d, f64, law, r, k) for law in (NORMAL, UNIFORM, KS) for r in rates for k in kinds)
