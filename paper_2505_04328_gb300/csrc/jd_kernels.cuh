@@ -2665,7 +2665,8 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
       return cudaGetLastError();
     }
   }
-  const bool chunk = fwd_chunks(form_key(D, sizeof(R) == 8, p->desc), mode == FWD_STORE ? SWEEP_STORE : SWEEP_PLAIN);
+  const bool chunk = fwd_chunks(form_key(D, sizeof(R) == 8, p->desc),
+                                mode & FWD_PAIR ? SWEEP_PAIR : mode == FWD_STORE ? SWEEP_STORE : SWEEP_PLAIN);
   switch (mode) {
     case FWD_COST:
       fwd_form<R, D, DU, FWD_COST>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr, nullptr, pc, jl,

@@ -18,12 +18,13 @@ struct FormKey {
   bool f64;
   bool one_jump;   // steps with one jump take the short path (one_jump of the kernels): the
                    // slot's words lie as compiled for D, and the law is additive for d > 2
+  bool ks;         // Keilson-Storer law
   double rate;     // jump_rate
 };
 inline FormKey form_key(int D, bool f64, const jd_problem_desc &q) {
   const bool packed = (q.d + 1) / 2 == (D + 1) / 2;
-  return FormKey{D, f64, packed && (D <= 2 || q.jump_law != JD_JUMP_KS),
-                 jump_rate(q.jump_law, q.lambda, q.T, q.Nt)};
+  const bool ks = q.jump_law == JD_JUMP_KS;
+  return FormKey{D, f64, packed && (D <= 2 || !ks), ks, jump_rate(q.jump_law, q.lambda, q.T, q.Nt)};
 }
 
 // Chunk length: the records hold a lane's jumps of a chunk but in rare chunks, and a pass of
@@ -33,24 +34,9 @@ inline int fwd_chunk_len(double rate, int most) {
   return n < most ? n : most;
 }
 
-// Whether a sweep takes its steps in chunks, by the jump rate per step.  The store sweep and
-// every FP64 sweep gain or tie at any rate; the other FP32 sweeps pay about 6% for the
-// chunks' passes without jumps and gain from about lambda dt = 0.005 on.  One launch at M =
-// 2^20, N_t = 160, d = 2 FP32, step by step -> in chunks, in ms:
-//   lambda dt          0            0.002         0.01          0.05          0.2           0.4
-//   cost          0.91 -> 0.97  1.01 -> 1.06  1.32 -> 1.23  2.33 -> 1.94  5.88 -> 3.27  9.96 -> 7.08
-//   store         1.11 -> 1.04  1.21 -> 1.15  1.56 -> 1.38  2.66 -> 2.24  6.38 -> 3.83  10.5 -> 8.48
-//   checkpoints   0.94 -> 0.99  1.02 -> 1.09  1.32 -> 1.25  2.30 -> 1.97  5.97 -> 3.34  10.1 -> 7.55
-//   store, pair   1.25 -> 1.22  1.38 -> 1.39  1.82 -> 1.79  4.16 -> 3.03  12.9 -> 6.65  21.9 -> 15.7
-//   ckpt., pair   1.11 -> 1.15  1.21 -> 1.27  1.59 -> 1.51  3.16 -> 2.44  10.1 -> 4.69  18.4 -> 11.9
-//   recompute     1.26 -> 1.35  1.39 -> 1.47  1.80 -> 1.70  3.18 -> 2.75  12.1 -> 12.1  23.7 -> 22.1
-//   adjoint (replay)
-// (double precision, M = 2^15: store sweep 1.17 -> 1.17, 1.30 -> 1.28, 1.68 -> 1.49, 2.68 ->
-// 2.17, 4.32 -> 4.14 ms up to 0.2.)  Between 0.004 and 0.007 the forms are within 3%.
-constexpr double FWD_CHUNK_RATE = 0.006;
-// What a launch runs: a sweep without stored states, the single store sweep, the replay of the
-// recompute adjoint.
-enum SweepKind { SWEEP_PLAIN, SWEEP_STORE, SWEEP_REPLAY };
+// What a launch runs: a single sweep without stored states (cost, checkpoints), the single store
+// sweep, a paired sweep, the replay of the recompute adjoint.
+enum SweepKind { SWEEP_PLAIN, SWEEP_STORE, SWEEP_PAIR, SWEEP_REPLAY };
 
 // d > 2: whether a one-jump step's slot draws are the whole warp's (coop_slot0_draws).  A lane
 // alone draws with its warp waiting; the warp-wide form costs the steps without jumps a
@@ -74,10 +60,41 @@ inline bool coop_slots(const FormKey &f, SweepKind kind) {
   return kind == SWEEP_REPLAY ? f.rate > 0.003 && f.rate <= 0.08 : f.rate > 0.01 && f.rate <= 0.03;
 }
 
+// d <= 2: whether a sweep takes its steps in chunks, by the jump rate per step.  The chunks'
+// passes cost a little where almost nothing jumps, and at high rates most jump steps have three
+// jumps or more and go to the general routine either way.  One launch at N_t = 160, step by
+// step -> in chunks, in ms (FP32 M = 2^18, the rates up to 0.01 of d = 1 and 2 at 2^20; FP64 2^15):
+//   lambda dt              0             0.002         0.006         0.1           0.3           0.5           0.6
+//   FP32 d = 1  cost       0.85 -> 0.85  0.95 -> 0.98  1.12 -> 1.09  0.96 -> 0.62  2.32 -> 1.30  3.12 -> 2.52  3.37 -> 3.10
+//               ckpt.      0.83 -> 0.88  0.93 -> 1.00  1.10 -> 1.11  0.95 -> 0.63  2.34 -> 1.31  3.16 -> 2.50  3.42 -> 3.09
+//               store      1.07 -> 0.87  1.17 -> 1.03  1.36 -> 1.19  1.06 -> 0.70  2.46 -> 1.47  3.24 -> 2.66  3.50 -> 3.22
+//               pair       0.94 -> 0.90  1.05 -> 1.06  0.35 -> 0.33  1.45 -> 0.77  4.35 -> 2.18  6.13 -> 4.26  6.66 -> 5.46
+//               replay     1.08 -> 1.09  1.19 -> 1.19  1.40 -> 1.29  1.25 -> 1.19  4.14 -> 3.90  5.95 -> 5.82  6.57 -> 6.55
+//   FP32 d = 2  cost       0.93 -> 0.89  1.02 -> 0.99  1.18 -> 1.08  0.94 -> 0.62  2.31 -> 1.35  3.11 -> 2.58  3.36 -> 3.21
+//               store      1.12 -> 0.98  1.22 -> 1.10  1.40 -> 1.22  1.05 -> 0.73  2.44 -> 1.68  3.23 -> 3.06  3.47 -> 3.71
+//               pair       1.08 -> 1.09  1.19 -> 1.21  0.38 -> 0.37  1.40 -> 0.85  4.11 -> 2.42  5.68 -> 4.89  6.19 -> 6.21
+//               replay     1.27 -> 1.25  1.41 -> 1.36  1.64 -> 1.49  1.45 -> 1.54  4.98 -> 5.22  7.30 -> 7.27  8.12 -> 7.99
+//   FP64 d = 1  store      0.61 -> 0.61  0.74 -> 0.70  0.93 -> 0.75  2.38 -> 1.61  4.12 -> 3.08  5.03 -> 4.82  5.36 -> 5.67
+//   FP64 d = 2  store      0.81 -> 0.79  0.91 -> 0.89  1.09 -> 0.99  2.46 -> 2.02  4.04 -> 4.07  4.83 -> 5.35  5.13 -> 5.84
+//               replay     1.05 -> 1.05  1.19 -> 1.18  1.41 -> 1.32  3.23 -> 2.87  6.76 -> 6.90  8.76 -> 9.30  9.49 -> 10.2
+//   FP64 KS     store      0.71 -> 0.79  0.84 -> 0.89  1.04 -> 0.96  2.68 -> 1.94  4.73 -> 4.42  5.79 -> 5.92  6.19 -> 6.48
+// (The FP32 replay of d = 2 also takes 0.73 -> 0.58 at 0.03, 3.95 -> 3.78 at 0.07 and 12.1 -> 13.4
+// at 0.2, M = 2^20; at 1.2 the FP32 store sweep of d = 2 takes 4.6 -> 6.3.)
+inline bool chunk_steps(const FormKey &f, SweepKind kind) {
+  double lo = 0.0, hi = 0.5;
+  if (f.f64) {
+    if (f.D == 2) hi = 0.3;
+    if (f.ks && kind != SWEEP_REPLAY) lo = 0.004;
+  } else {
+    if (f.D == 2 && kind == SWEEP_REPLAY) hi = 0.08;
+    if (f.D == 1 && kind == SWEEP_PLAIN) lo = 0.005;
+  }
+  return f.rate >= lo && f.rate <= hi;
+}
+
 // The form of a forward sweep or replay: in chunks (d <= 2) or with warp-wide slot draws (d > 2).
 inline bool fwd_chunks(const FormKey &f, SweepKind kind) {
-  if (f.D > 2) return coop_slots(f, kind);
-  return f.f64 || kind == SWEEP_STORE || f.rate > FWD_CHUNK_RATE;
+  return f.D > 2 ? coop_slots(f, kind) : chunk_steps(f, kind);
 }
 
 // Parameter gradients: the jump draws are kept up to this jump rate per step; beyond it a

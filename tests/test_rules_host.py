@@ -8,7 +8,7 @@ import pytest
 from paper_2505_04328_gb300 import _build
 
 NONE, NORMAL, UNIFORM, KS = range(4)
-PLAIN, STORE, REPLAY = range(3)
+PLAIN, STORE, PAIR, REPLAY = range(4)
 
 SRC = r"""
 #include "jd_rules.h"
@@ -95,3 +95,32 @@ def test_warp_wide_draws_need_a_one_jump_path(rules, f64):
         assert any(rules.chunks(d, f64, NORMAL, r, k) for r in rates for k in kinds)
     for d in (5, 6):
         assert not any(rules.chunks(d, f64, law, r, k) for law in (NORMAL, UNIFORM, KS) for r in rates for k in kinds)
+
+
+# (d, f64, law, kind, rate, in chunks): beside each line the launch step by step -> in chunks, ms
+CHUNKS = [
+    (2, False, UNIFORM, REPLAY, 0.07, True),    # 3.95 -> 3.78
+    (2, False, UNIFORM, REPLAY, 0.1, False),    # 5.26 -> 5.68
+    (2, False, KS, REPLAY, 0.2, False),         # 12.6 -> 14.5
+    (1, False, NORMAL, REPLAY, 0.3, True),      # 14.8 -> 14.2
+    (2, False, UNIFORM, STORE, 0.5, True),      # 3.23 -> 3.06
+    (2, False, UNIFORM, STORE, 0.8, False),     # 3.87 -> 4.82
+    (2, False, UNIFORM, PAIR, 0.8, False),      # 7.65 -> 9.41
+    (2, True, UNIFORM, PLAIN, 0.2, True),       # 3.22 -> 2.95
+    (2, True, UNIFORM, PLAIN, 0.4, False),      # 4.42 -> 4.71
+    (1, True, NORMAL, STORE, 0.4, True),        # 4.64 -> 4.04
+    (1, True, NORMAL, STORE, 0.8, False),       # 5.98 -> 6.81
+    (2, True, KS, STORE, 0.0, False),           # 0.71 -> 0.79
+    (2, True, KS, PAIR, 0.003, False),          # 1.17 -> 1.25
+    (2, True, KS, STORE, 0.006, True),          # 1.04 -> 0.96
+    (2, True, UNIFORM, STORE, 0.0, True),       # 0.81 -> 0.79
+    (1, False, NORMAL, PLAIN, 0.002, False),    # 0.945 -> 0.977
+    (1, False, NORMAL, PLAIN, 0.008, True),     # 1.20 -> 1.13
+    (2, False, UNIFORM, PLAIN, 0.0, True),      # 0.934 -> 0.894
+    (2, False, UNIFORM, PAIR, 0.003, True),     # 1.417 -> 1.365 stored
+]
+
+
+@pytest.mark.parametrize("d,f64,law,kind,rate,want", CHUNKS)
+def test_chunks_where_they_are_faster(rules, d, f64, law, kind, rate, want):
+    assert rules.chunks(d, f64, law, rate, kind) == want
