@@ -97,11 +97,21 @@ inline bool fwd_chunks(const FormKey &f, SweepKind kind) {
   return f.D > 2 ? coop_slots(f, kind) : chunk_steps(f, kind);
 }
 
-// Parameter gradients: the jump draws are kept up to this jump rate per step; beyond it a
-// segment's jumps outgrow the records and most steps have several (M = 2^19, N_t = 160, d = 2
-// FP32, regenerated -> kept: 0.80 -> 0.86 ms without jumps, 1.36 -> 0.94 at 0.002, 3.29 ->
-// 1.16 at 0.01, 7.82 -> 4.16 at 0.05, 10.9 -> 9.8 at 0.1, 16.0 -> 20.0 at 0.2).
-constexpr double THETA_KEEP_RATE = 0.12;
-inline bool theta_keeps(const FormKey &f) { return f.rate <= THETA_KEEP_RATE; }
+// Parameter gradients: whether the recompute adjoint keeps its jump steps' draws (adj_theta_body;
+// built for d <= 2 and FP32 d = 4).  Without jumps its passes cost a little; at high rates a
+// segment's jumps outgrow the records and most jump steps have several.  One launch at N_t =
+// 160, regenerated -> kept, in ms (FP32 d <= 2 M = 2^20, d = 4 2^17; FP64 2^15):
+//   lambda dt    0             0.0002        0.0005*       0.02          0.1           0.12          0.14          0.17
+//   FP32 d = 1   1.29 -> 1.33  1.39 -> 1.34  1.48 -> 1.36  7.63 -> 2.70  17.1 -> 15.1  18.7 -> 18.4  20.2 -> 21.7  22.4 -> 26.2
+//        d = 2   1.55 -> 1.56  1.66 -> 1.58  1.75 -> 1.59  9.01 -> 2.93  20.0 -> 17.6  21.8 -> 21.7  23.7 -> 25.7  26.3 -> 31.2
+//        KS      1.53 -> 1.55  1.66 -> 1.56  1.75 -> 1.58  9.72 -> 3.09  21.8 -> 20.4  24.0 -> 25.3  26.2 -> 30.0  29.2 -> 36.4
+//        d = 4   0.57 -> 0.64  0.60 -> 0.64  0.64 -> 0.64  5.01 -> 1.98  11.3 -> 11.6  12.6 -> 13.9  13.8 -> 16.0  15.3 -> 18.7
+//   FP64 d = 1   0.83 -> 0.83  0.93 -> 0.86  0.99 -> 0.87  3.57 -> 1.64  6.70 -> 4.85  7.22 -> 6.04  7.60 -> 6.82  8.17 -> 7.90
+//        d = 2   1.22 -> 1.22  1.31 -> 1.25  1.36 -> 1.27  3.89 -> 2.43  6.86 -> 5.50  7.33 -> 6.57  7.68 -> 7.34  8.14 -> 8.34
+// (* 0.0004; d = 4 at 0.07 9.16 -> 7.82.)
+inline bool theta_keeps(const FormKey &f) {
+  if (f.D > 2) return f.rate > 0.0004 && f.rate <= 0.09;
+  return f.rate > 0.0 && f.rate <= (f.f64 ? 0.16 : f.ks ? 0.11 : 0.12);
+}
 
 }  // namespace jd

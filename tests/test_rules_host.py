@@ -124,3 +124,24 @@ CHUNKS = [
 @pytest.mark.parametrize("d,f64,law,kind,rate,want", CHUNKS)
 def test_chunks_where_they_are_faster(rules, d, f64, law, kind, rate, want):
     assert rules.chunks(d, f64, law, rate, kind) == want
+
+
+# (d, f64, law, rate, kept): the recompute adjoint with parameter gradients, regenerated -> kept, ms
+KEPT = [
+    (1, False, NORMAL, 0.0, False),    # 1.29 -> 1.33
+    (2, False, NONE, 0.05, False),     # 1.55 -> 1.56
+    (2, False, UNIFORM, 0.0002, True),  # 1.66 -> 1.58
+    (4, False, NORMAL, 0.0002, False),  # 0.60 -> 0.64
+    (4, False, NORMAL, 0.002, True),   # 1.36 -> 0.65
+    (4, False, NORMAL, 0.1, False),    # 11.3 -> 11.6
+    (2, False, UNIFORM, 0.1, True),    # 20.0 -> 17.6
+    (2, False, KS, 0.12, False),       # 24.0 -> 25.3
+    (2, False, UNIFORM, 0.2, False),   # 28.7 -> 36.1
+    (2, True, UNIFORM, 0.14, True),    # 7.68 -> 7.34
+    (1, True, NORMAL, 0.2, False),     # 8.80 -> 8.85
+]
+
+
+@pytest.mark.parametrize("d,f64,law,rate,want", KEPT)
+def test_jump_draws_kept_where_that_is_faster(rules, d, f64, law, rate, want):
+    assert rules.keeps(d, f64, law, rate) == want
