@@ -47,6 +47,7 @@ struct KParams {
   // block; last in the struct, so kernels that do not read them see the same layout
   uint32_t rk0[10], rk1[10];
   int chunk;                      // steps per chunk of the chunked forward sweep (4, 8 or 16)
+  int ks_one;                     // Keilson-Storer steps with one jump take the short path
 };
 
 // Device buffers of one launch (unused ones are null).

@@ -257,14 +257,14 @@ __host__ __device__ constexpr int seg_len() {
 // Steps with one jump take a short path (the common case); two or more go through
 // build_jump_step.  The short path takes every law for d <= 2 (Keilson-Storer steps all went
 // through build_jump_step before: 5.26 -> 4.13 ms per store sweep at M = 2^20, N_t = 500,
-// lambda dt = 0.0036, where 11% of the warp-steps have a jump), the additive laws for larger
-// d (whose sweeps ran 1% slower with the law's branch).
+// lambda dt = 0.0036, where 11% of the warp-steps have a jump; up to the rate of ks_one_jump),
+// the additive laws for larger d (whose sweeps ran 1% slower with the law's branch).
 template <int D>
 constexpr bool ONE_JUMP_KS = D <= 2;
 // The step has exactly one jump and its slot words lie as compiled (the one-jump paths).
 template <typename R, int D, int DU>
 __device__ __forceinline__ bool one_jump(const KParams<R, D, DU> &kp, uint32_t w0) {
-  return (ONE_JUMP_KS<D> || kp.jump_law != JD_JUMP_KS) && kp.npair == MainWords<D>::PD &&
+  return (kp.jump_law != JD_JUMP_KS || (ONE_JUMP_KS<D> && kp.ks_one)) && kp.npair == MainWords<D>::PD &&
          (unsigned long long)w0 < kp.thr[1];
 }
 
@@ -281,8 +281,11 @@ __device__ __forceinline__ void apply_one_jump(const KParams<R, D, DU> &kp, R (&
   }
 }
 
-// The one-jump step out of line: sub-step to the jump, jump, sub-step to t_{k+1}.  x is
-// updated in place; y1 receives the post-jump state; returns the jump's time fraction.
+// The one-jump step out of line (additive laws: where the parameter-gradient adjoint's replay
+// takes it, at high jump rates, Keilson-Storer steps are faster all through build_jump_step:
+// 8.53 -> 7.62 ms per launch at M = 2^18, N_t = 160, lambda dt = 0.2, 12.0 -> 10.2 at 0.4):
+// sub-step to the jump, jump, sub-step to t_{k+1}.  x is updated in place; y1 receives the
+// post-jump state; returns the jump's time fraction.
 template <typename R, int D, int DU>
 __device__ __noinline__ R one_jump_substeps(const KParams<R, D, DU> &kp, int k, uint32_t m, const R *z,
                                             const R *uk, R *x, R *y1) {
@@ -438,7 +441,7 @@ __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, cons
     plain_update(kh, f, z, x);
     return 0;
   }
-  if (!INLINE_JUMP && one_jump(kp, w0)) {
+  if (!INLINE_JUMP && kp.jump_law != JD_JUMP_KS && one_jump(kp, w0)) {
     // copies: an address taken of x or uk themselves would move them to local memory
     R zc[D], xc[D], uc[DU], y1[D];
 #pragma unroll
@@ -2569,6 +2572,7 @@ void make_kparams(const jd_problem *p, int64_t m_begin, int64_t mloc, KParams<R,
   kp.chunk = 4;
   if constexpr (fwd_chunked<D>())
     kp.chunk = fwd_chunk_len(jump_rate(q.jump_law, q.lambda, q.T, q.Nt), FwdChunk<R, D>::CH);
+  kp.ks_one = ks_one_jump(jump_rate(q.jump_law, q.lambda, q.T, q.Nt));
   kp.S = p->S;   // checkpoint spacing of the recompute plan (a power of two, 16 .. 64)
   kp.nblk = (int)ceil_div(mloc, TPB);
   kp.m_begin = q.m_offset + m_begin;   // global path index (a shard starts at m_offset)

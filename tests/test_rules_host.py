@@ -31,6 +31,7 @@ int chunk_len(int d, int law, double rate, int most) { return fwd_chunk_len(key(
 int chunks(int d, int f64, int law, double rate, int kind) {
   return fwd_chunks(key(d, f64, law, rate), (SweepKind)kind);
 }
+int ks_short(double rate) { return ks_one_jump(rate); }
 int keeps(int d, int f64, int law, double rate) { return theta_keeps(key(d, f64, law, rate)); }
 }
 """
@@ -60,6 +61,10 @@ def rules(tmp_path_factory):
         @staticmethod
         def chunks(d, f64, law, rate, kind):
             return bool(so.chunks(d, int(f64), law, ctypes.c_double(rate), kind))
+
+        @staticmethod
+        def ks_short(rate):
+            return bool(so.ks_short(ctypes.c_double(rate)))
 
         @staticmethod
         def keeps(d, f64, law, rate):
@@ -145,3 +150,9 @@ KEPT = [
 @pytest.mark.parametrize("d,f64,law,rate,want", KEPT)
 def test_jump_draws_kept_where_that_is_faster(rules, d, f64, law, rate, want):
     assert rules.keeps(d, f64, law, rate) == want
+
+
+def test_keilson_storer_short_path_ends_at_high_rates(rules):
+    """FP32 store sweep, all steps by the general routine -> with the short path: 1.93 -> 1.16
+    ms at 0.2, 3.24 -> 3.59 at 0.55."""
+    assert rules.ks_short(0.2) and not rules.ks_short(0.55)
