@@ -52,18 +52,23 @@ enum SweepKind { SWEEP_PLAIN, SWEEP_STORE, SWEEP_PAIR, SWEEP_REPLAY };
 //   FP32 d = 8  M = 200,003  cost    0.65 -> 0.67   0.75 -> 0.71   1.04 -> 0.87   2.45 -> 1.78
 //                            store   0.71 -> 0.78   0.80 -> 0.83   1.13 -> 1.01   2.51 -> 2.22
 //                            replay  1.04 -> 1.08   1.37 -> 1.20   2.81 -> 2.00   6.24 -> 5.08
-//   FP32 d = 4               cost    0.34 -> 0.37   0.38 -> 0.40   0.50 -> 0.50   0.89 -> 0.94
+//   FP32 d = 4               cost    0.34 -> 0.37   0.38 -> 0.40   0.51 -> 0.50   0.89 -> 0.94
 //                            replay  0.57 -> 0.57   0.63 -> 0.61   0.81 -> 0.76   1.76 -> 1.57
 //   FP64 d = 8  M = 16,000   store   1.86 -> 1.86   2.20 -> 2.00   3.08 -> 2.50   5.63 -> 4.20
 //   FP64 d = 4               store   0.87 -> 0.88   1.02 -> 0.94   1.44 -> 1.20   2.53 -> 2.15
-// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)  Where no
+// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)  The FP32
+// d = 4 cost and checkpoint sweeps gain between 0.01 and 0.03: cost 0.506 -> 0.499 ms at 0.01,
+// 0.571 -> 0.552 at 0.015, 0.632 -> 0.609 at 0.02, 0.735 -> 0.719 at 0.03 (M = 50,001: 0.161 ->
+// 0.161, 0.184 -> 0.181, 0.204 -> 0.203); its store sweep not for every size: 0.718 -> 0.700 at
+// 0.02, but 0.186 -> 0.190 at 0.01 and 0.271 -> 0.281 at 0.03 for M = 50,001.  Where no
 // step takes the one-jump path the form only costs: Keilson-Storer d = 8, FP32, M = 2^17, store
 // sweep 1.17 -> 1.33 ms at 0.01, 1.52 -> 1.83 at 0.02, cost 1.07 -> 1.17 and 1.47 -> 1.63.
 inline bool coop_slots(const FormKey &f, SweepKind kind) {
   if (!f.one_jump) return false;
   if (f.f64) return f.rate > 0.0005 && f.rate <= 0.1;
   if (f.D == 8) return f.rate > (kind == SWEEP_STORE ? 0.005 : 0.0015) && f.rate <= 0.08;
-  return kind == SWEEP_REPLAY ? f.rate > 0.003 && f.rate <= 0.08 : f.rate > 0.01 && f.rate <= 0.03;
+  if (kind == SWEEP_REPLAY) return f.rate > 0.003 && f.rate <= 0.08;
+  return kind == SWEEP_PLAIN && f.rate > 0.01 && f.rate <= 0.025;
 }
 
 // d <= 2: whether a sweep takes its steps in chunks, by the jump rate per step.  The chunks'

@@ -156,3 +156,13 @@ def test_keilson_storer_short_path_ends_at_high_rates(rules):
     """FP32 store sweep, all steps by the general routine -> with the short path: 1.93 -> 1.16
     ms at 0.2, 3.24 -> 3.59 at 0.55."""
     assert rules.ks_short(0.2) and not rules.ks_short(0.55)
+
+
+def test_four_components_draw_warp_wide_where_that_gains(rules):
+    """FP32 d = 4: the store sweep gains at no rate for every size (M = 50,001 at 0.03: 0.271 ->
+    0.281 ms), the cost and checkpoint sweeps around 0.02, the replay in a wide range."""
+    for rate in (0.008, 0.012, 0.02, 0.03, 0.05):
+        assert not rules.chunks(4, False, NORMAL, rate, STORE)
+        assert rules.chunks(4, False, NORMAL, rate, REPLAY)
+    assert rules.chunks(4, False, NORMAL, 0.02, PLAIN)
+    assert not rules.chunks(4, False, NORMAL, 0.03, PLAIN) and not rules.chunks(4, False, NORMAL, 0.009, PLAIN)
