@@ -590,7 +590,7 @@ static size_t base_bytes(const jd_problem_desc &q, int D, int DU, size_t es) {
   return (size_t)q.Nt * DU * es + (size_t)(q.Nt + 1) * D * es + 4 * nu * 8 + NSCAL * 8 + nblk * 8 +
          (size_t)q.Nt * DU * grad_parts(q.M) * 8 + (size_t)(D + 2) * nblk * 8 +
          (size_t)ceil_div(q.M, JD_UNIT_PATHS) * (1 + nu) * 8 +
-         (pre_pass(q, es) ? pre_bytes(q.Nt, D, q.M, es) : 0) +
+         (pre_pass(q, D, es) ? pre_bytes(q.Nt, D, q.M, es) : 0) +
          (D == 32 ? 16384 + (size_t)q.Nt * 32 * sizeof(float) : 0);
 }
 
@@ -1571,7 +1571,7 @@ jd_status jd::create_problem(const jd_problem_desc &q, const jd::ProblemOpts &op
   ALLOC(p->partG, (size_t)q.Nt * p->DU * grad_parts(q.M) * 8, "gradient partials");
   ALLOC(p->partT, (size_t)(p->D + 2) * p->nblk * 8, "parameter partials");
   ALLOC(p->units, (size_t)n_units(q.M) * (1 + nu) * 8, "unit sums");
-  if (!opts.no_pre && pre_pass(q, es)) {   // a small problem: the draws' pre-pass buffers
+  if (!opts.no_pre && pre_pass(q, p->D, es)) {   // a small problem: the draws' pre-pass buffers
     ALLOC(p->pre_w, (size_t)q.Nt * q.M * 4, "pre-drawn Poisson words");
     ALLOC(p->pre_z, pre_z_values(q.Nt, p->D, q.M) * es, "pre-drawn normals and slot draws");
     ALLOC(p->pre_key, sizeof(unsigned long long), "pre-drawn key");

@@ -139,24 +139,6 @@ inline int ring_lanes(int N) {
 }
 constexpr int RING_MAX = 2048;   // 8 blocks of 256 lanes: the largest portable cluster
 
-// Draw pre-pass: a problem with d <= 2 of few paths (its sweeps are latency-bound: each
-// thread's steps are a chain of dependent operations, and the Philox and Box-Muller of every
-// step sit on that chain) takes its main-stream draws in one parallel kernel first, when
-// their buffers stay small.  Its sweeps then run few lanes per warp (SPREAD_LANES), which
-// costs them instruction issue as the paths grow: the limits are where three projected-
-// gradient iterations take as long with the chunked sweeps (N_t = 200, pre-drawn / chunked
-// in us, by lambda dt):
-//                          0.002         0.02          0.1
-//   FP32 d = 1  M = 8000   746 / 597     902 / 854     1489 / 1565
-//               M = 10000  820 / 587     999 / 848     1627 / 1562
-//   FP64 d = 1  M = 7500   2863 / 2839   3464 / 3856   5909 / 6436
-//               M = 9000   3337 / 2845   3982 / 3851   7063 / 6409
-//   FP64 d = 2  M = 6000   4358 / 4022   5200 / 5394   7924 / 8960
-//               M = 7500   5387 / 4014   6401 / 5407   9792 / 8967
-inline int64_t pre_max_paths(int D, size_t es, double lamdt) {
-  if (es == 4) return lamdt > 0.05 ? 152 * 64 : 152 * 40;
-  return D == 1 ? 152 * 56 : 152 * 40;
-}
 constexpr size_t PRE_MAX_BYTES = (size_t)128 << 20;
 // pre_z holds the normals, the slot-0 draws and then the paths' cost pairs of the sweeps
 // (2 controls x M pairs of 2 values)
@@ -167,12 +149,10 @@ inline size_t pre_bytes(int Nt, int D, int64_t M, size_t es) {
   // words; normals, slot-0 draws and cost pairs; the key of the draws held
   return (size_t)Nt * (size_t)M * 4 + pre_z_values(Nt, D, M) * es + sizeof(unsigned long long);
 }
-inline bool pre_pass(const jd_problem_desc &q, size_t es) {
-  const int d = q.d, Nt = q.Nt;
-  const int64_t M = q.M;
-  const double lamdt = jump_rate(q.jump_law, q.lambda, q.T, Nt);
-  const int D = d <= 1 ? 1 : 2;
-  return d <= 2 && M <= pre_max_paths(D, es, lamdt) && pre_bytes(Nt, D, M, es) <= PRE_MAX_BYTES;
+// Whether a problem of the compiled dimension D keeps the pre-pass buffers: it may come below
+// pre_max_paths, whose limit follows the jump rate (jd_problem_update changes it).
+inline bool pre_pass(const jd_problem_desc &q, int D, size_t es) {
+  return D <= 2 && q.M <= pre_top_paths(D, es == 8) && pre_bytes(q.Nt, D, q.M, es) <= PRE_MAX_BYTES;
 }
 
 struct FbBufs {

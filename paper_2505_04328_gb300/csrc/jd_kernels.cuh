@@ -2629,8 +2629,14 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
     p2 = PairOut<R, D>{static_cast<const R *>(b.uk2), b.partC2, static_cast<R *>(b.traj2), static_cast<R *>(b.ckpt2),
                        JLog<R, D>{static_cast<typename V2<R>::T *>(b.log_kt2), static_cast<R *>(b.log_y2), mloc,
                                   b.log_cap}};
+  const FormKey form = form_key(D, sizeof(R) == 8, p->desc);
+  const SweepKind kind = mode & FWD_PAIR ? (mode & FWD_STORE ? SWEEP_STORE_PAIR : SWEEP_CKPT_PAIR)
+                         : mode == FWD_STORE ? SWEEP_STORE
+                         : mode == FWD_COST  ? SWEEP_COST
+                                             : SWEEP_CKPT;
   if constexpr (D <= 2) {
-    if (b.pre_w) {   // a small problem: all main-stream draws in one parallel pass first
+    // a small problem: all main-stream draws in one parallel pass first
+    if (b.pre_w && p->desc.M <= pre_max_paths(form, kind)) {
       R *pz = static_cast<R *>(b.pre_z), *ps = pz + (size_t)kp.Nt * D * mloc;
       Pair<R> *cw = reinterpret_cast<Pair<R> *>(ps + (size_t)kp.Nt * (1 + 2 * D) * mloc);
       const unsigned long long key = draws_key(kp, mloc);
@@ -2669,8 +2675,7 @@ cudaError_t op_fwd(const jd_problem *p, int mode, int64_t m_begin, int64_t mloc,
       return cudaGetLastError();
     }
   }
-  const bool chunk = fwd_chunks(form_key(D, sizeof(R) == 8, p->desc),
-                                mode & FWD_PAIR ? SWEEP_PAIR : mode == FWD_STORE ? SWEEP_STORE : SWEEP_PLAIN);
+  const bool chunk = fwd_chunks(form, kind);
   switch (mode) {
     case FWD_COST:
       fwd_form<R, D, DU, FWD_COST>(chunk)<<<grid, TPB, 0, s>>>(kp, u, xd, b.partC, nullptr, nullptr, nullptr, pc, jl,

@@ -142,7 +142,7 @@ static jd_status noalloc_run(const jd_problem_desc &q, unsigned char *scratch, c
   KParams<R, D, 1> kp;
   noalloc_kparams<R, D, 1>(q, kp);
   const JLog<R, D> nolog{nullptr, nullptr, M, 0};
-  const auto k = fwd_form<R, D, 1, FWD_COST>(fwd_chunks(form_key(D, sizeof(R) == 8, q), SWEEP_PLAIN));
+  const auto k = fwd_form<R, D, 1, FWD_COST>(fwd_chunks(form_key(D, sizeof(R) == 8, q), SWEEP_COST));
   k<<<(unsigned)nblk, TPB, 0, s>>>(kp, uk, xdk, partC, nullptr, nullptr, nullptr, nullptr, nolog, nullptr, M,
                                    PairOut<R, D>{}, PreDraws<R, D>{});
   noalloc_finalize_kernel<<<1, 256, 0, s>>>(partC, nblk, u, Nt, 0.5 * q.nu * (q.T / Nt), 1.0 / (double)M, J);

@@ -2,6 +2,8 @@
 // jump law and jump rate.  Plain C++ without CUDA, so that any host can check them.
 #pragma once
 
+#include <cstdint>
+
 #include "jd.h"
 
 namespace jd {
@@ -40,9 +42,9 @@ inline int fwd_chunk_len(double rate, int most) {
   return n < most ? n : most;
 }
 
-// What a launch runs: a single sweep without stored states (cost, checkpoints), the single store
-// sweep, a paired sweep, the replay of the recompute adjoint.
-enum SweepKind { SWEEP_PLAIN, SWEEP_STORE, SWEEP_PAIR, SWEEP_REPLAY };
+// What a launch runs: a forward sweep (cost, checkpoints, stored states; the last two also for a
+// pair of controls) or the replay of the recompute adjoint.
+enum SweepKind { SWEEP_COST, SWEEP_CKPT, SWEEP_STORE, SWEEP_STORE_PAIR, SWEEP_CKPT_PAIR, SWEEP_REPLAY };
 
 // d > 2: whether a one-jump step's slot draws are the whole warp's (coop_slot0_draws).  A lane
 // alone draws with its warp waiting; the warp-wide form costs the steps without jumps a
@@ -68,7 +70,7 @@ inline bool coop_slots(const FormKey &f, SweepKind kind) {
   if (f.f64) return f.rate > 0.0005 && f.rate <= 0.1;
   if (f.D == 8) return f.rate > (kind == SWEEP_STORE ? 0.005 : 0.0015) && f.rate <= 0.08;
   if (kind == SWEEP_REPLAY) return f.rate > 0.003 && f.rate <= 0.08;
-  return kind == SWEEP_PLAIN && f.rate > 0.01 && f.rate <= 0.025;
+  return (kind == SWEEP_COST || kind == SWEEP_CKPT) && f.rate > 0.01 && f.rate <= 0.025;
 }
 
 // d <= 2: whether a sweep takes its steps in chunks, by the jump rate per step.  The chunks'
@@ -98,7 +100,7 @@ inline bool chunk_steps(const FormKey &f, SweepKind kind) {
     if (f.ks && kind != SWEEP_REPLAY) lo = 0.004;
   } else {
     if (f.D == 2 && kind == SWEEP_REPLAY) hi = 0.08;
-    if (f.D == 1 && kind == SWEEP_PLAIN) lo = 0.005;
+    if (f.D == 1 && (kind == SWEEP_COST || kind == SWEEP_CKPT)) lo = 0.005;
   }
   return f.rate >= lo && f.rate <= hi;
 }
@@ -107,6 +109,53 @@ inline bool chunk_steps(const FormKey &f, SweepKind kind) {
 inline bool fwd_chunks(const FormKey &f, SweepKind kind) {
   return f.D > 2 ? coop_slots(f, kind) : chunk_steps(f, kind);
 }
+
+// Draw pre-pass: a problem with d <= 2 of few paths (its sweeps are latency-bound: each
+// thread's steps are a chain of dependent operations, and the Philox and Box-Muller of every
+// step sit on that chain) takes its main-stream draws in one parallel kernel first, when
+// their buffers stay small.  Its sweeps then run few lanes per warp (SPREAD_LANES), which costs
+// them instruction issue as the paths grow (a pair's two controls are sweeps of their own), and
+// save more where more steps jump.  The limits per kind of sweep and jump rate lie below the path
+// count from which the other form is faster; that count, measured at N_t = 200 with the draws held
+// (Keilson-Storer as d = 2 where it is not given):
+//   lambda dt          0       0.002   0.007   0.015   0.03    0.07    0.2
+//   FP32 cost   d = 1  7200    7800    7500    10800   11300   13000+  13000+
+//               d = 2  3800    5000    7000    9100    10200   11000   11000
+//        ckpt.  d = 1  7400    7800    6300    10200   10700   13000+  13000+
+//               d = 2  none    none    2900    5500    7900    10200   10600
+//        store  d = 1  none    none    3500    8100    9600    10700   12100
+//               d = 2  none    none    4800    8900    8400    10500   13000+
+//        store, d = 1  none    none    2600    5100    6900    8300    10400
+//        pair   d = 2  none    1100    2500    5100    7000    8200    10400
+//        ckpt., d = 1  none    3100    5000    7700    8500    9900    11200
+//        pair   d = 2  1200    1800    3700    5600    7600    9000    10400
+//   FP64 single d = 1  9300    10100   10600   10900   11300   11700   10200
+//               d = 2  6100    6800    7200    7600    7900    8400    9700
+//        pair   d = 1  6000    6500    6900    7200    7400    7400    7200
+//               d = 2  4100    4600    5000    5300    5700    6000    6300
+//               KS     5000    5900    6300    6300    6400    6400    6600
+// ("none": the other form is faster at 1000 paths already: FP32 d = 1 store sweep of 3000 paths
+// at 0.0005 45 against 58 us, its pair 48 against 74.)
+inline int64_t pre_max_paths(const FormKey &f, SweepKind kind) {
+  if (f.D > 2) return 0;
+  // multiples of 152 paths (an SM's share) by rate: below 0.004, 0.01, 0.02, 0.05, 0.1, above
+  static const unsigned char f32[5][2][6] = {
+      {{40, 40, 64, 64, 64, 64}, {24, 40, 56, 64, 64, 64}},    // cost: d = 1, d = 2
+      {{40, 40, 64, 64, 64, 64}, {0, 16, 32, 48, 64, 64}},     // checkpoints
+      {{0, 20, 48, 56, 64, 64}, {0, 28, 52, 52, 64, 64}},      // store
+      {{0, 16, 32, 44, 52, 64}, {0, 16, 32, 44, 52, 64}},      // store, pair
+      {{16, 32, 48, 52, 64, 64}, {8, 24, 36, 48, 56, 64}}};    // checkpoints, pair
+  const int c = f.rate < 0.004 ? 0 : f.rate < 0.01 ? 1 : f.rate < 0.02 ? 2 : f.rate < 0.05 ? 3 : f.rate < 0.1 ? 4 : 5;
+  if (f.f64) {
+    if (kind != SWEEP_STORE_PAIR && kind != SWEEP_CKPT_PAIR) return 152 * (f.D == 1 ? 56 : 40);
+    static const unsigned char pair[3][6] = {
+        {40, 44, 44, 48, 48, 46}, {28, 32, 32, 32, 36, 40}, {32, 40, 40, 40, 40, 40}};   // d = 1, d = 2, KS
+    return 152 * (int64_t)pair[f.ks && f.D == 2 ? 2 : f.D - 1][c];
+  }
+  return 152 * (int64_t)f32[kind][f.D - 1][c];
+}
+// The largest of the limits.
+inline int64_t pre_top_paths(int D, bool f64) { return D > 2 ? 0 : 152 * (!f64 ? 64 : D == 1 ? 56 : 40); }
 
 // Parameter gradients: whether the recompute adjoint keeps its jump steps' draws (adj_theta_body;
 // built for d <= 2 and FP32 d = 4).  Without jumps its passes cost a little; at high rates a

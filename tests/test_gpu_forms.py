@@ -5,7 +5,7 @@ import pytest
 
 import oracle
 import workloads
-from paper_2505_04328_gb300 import JdProblem, build
+from paper_2505_04328_gb300 import JdProblem, build, launch_count
 
 pytestmark = pytest.mark.gpu
 
@@ -39,3 +39,53 @@ def test_keilson_storer_sweeps_across_the_rates(prec, lamdt):
         r = oracle.path(p, u, m)
         assert abs(c[m] - r["cost"]) <= tol * abs(r["cost"])
         assert np.max(np.abs(X[m, -1] - r["X"][-1])) <= tol * max(1.0, np.max(np.abs(r["X"][-1])))
+
+
+def _launches(f):
+    n = launch_count()
+    out = f()
+    return out, launch_count() - n
+
+
+# a pre-drawn cost evaluation launches the draws and the combination of the paths' costs beside
+# the sweep
+PRE_EXTRA = 2
+
+
+@pytest.mark.parametrize("d", [1, 2])
+def test_form_follows_the_rate_of_an_update(d):
+    """The path limit of the FP32 pre-drawn cost sweep rises with the jump rate: a problem
+    between the limits moves between the forms as its rate is updated, with a fresh problem's
+    bits."""
+    M, Nt = 6500, 40
+    p = (workloads.lq_scalar if d == 1 else workloads.double_well)(M=M, Nt=Nt)
+    u = workloads.random_control(p, seed=3, scale=0.6)
+    low, high = p.replace(lam=0.001 * Nt / p.T), p.replace(lam=0.1 * Nt / p.T)
+    with JdProblem(low) as jp:
+        J0, n0 = _launches(lambda: jp.cost(u))
+        jp.update(high)
+        J1, n1 = _launches(lambda: jp.cost(u))
+        g1 = jp.gradient(u)[1]
+        jp.update(low)
+        J2, n2 = _launches(lambda: jp.cost(u))
+    assert n1 == n0 + PRE_EXTRA and n2 == n0 and J2 == J0
+    with JdProblem(high) as jp:
+        J3, n3 = _launches(lambda: jp.cost(u))
+        assert n3 == n1 and J3 == J1 and np.array_equal(jp.gradient(u)[1], g1)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("law", [workloads.JUMP_NORMAL, workloads.JUMP_UNIFORM, workloads.JUMP_KS])
+@pytest.mark.parametrize("Nt,lamdt", [(33, 0.0), (61, 0.003), (40, 0.02), (35, 0.3), (17, 0.7)])
+def test_pre_drawn_sweeps_equal_the_others(law, prec, Nt, lamdt):
+    """The last shard of a problem is small enough for the pre-drawn sweeps at every rate, the
+    whole is not: which form ran shows in the launches, and the units' sums are equal."""
+    p = workloads.double_well(M=16384 + 3001, Nt=Nt).replace(lam=lamdt * Nt / 2.0, seed=11, jump_law=law, jump_gain=0.5)
+    u = workloads.random_control(p, seed=3, scale=0.6)
+    with JdProblem(p, prec=prec, mode="stored") as jp:
+        whole, n = _launches(lambda: jp.cost_units(u))
+        grads = jp.gradient_units(u)
+    with JdProblem(p.replace(M=3001, m_offset=16384), prec=prec, mode="stored") as jp:
+        part, npart = _launches(lambda: jp.cost_units(u))
+        assert np.array_equal(grads[1:], jp.gradient_units(u))
+    assert npart == n + PRE_EXTRA and np.array_equal(whole[1:], part)

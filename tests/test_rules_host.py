@@ -8,7 +8,7 @@ import pytest
 from paper_2505_04328_gb300 import _build
 
 NONE, NORMAL, UNIFORM, KS = range(4)
-PLAIN, STORE, PAIR, REPLAY = range(4)
+COST, CKPT, STORE, PAIR, CKPT_PAIR, REPLAY = range(6)
 
 SRC = r"""
 #include "jd_rules.h"
@@ -31,6 +31,10 @@ int chunk_len(int d, int law, double rate, int most) { return fwd_chunk_len(key(
 int chunks(int d, int f64, int law, double rate, int kind) {
   return fwd_chunks(key(d, f64, law, rate), (SweepKind)kind);
 }
+long long pre_max(int d, int f64, int law, double rate, int kind) {
+  return pre_max_paths(key(d, f64, law, rate), (SweepKind)kind);
+}
+long long pre_top(int d, int f64) { return pre_top_paths(d, f64 != 0); }
 int ks_short(double rate) { return ks_one_jump(rate); }
 int keeps(int d, int f64, int law, double rate) { return theta_keeps(key(d, f64, law, rate)); }
 }
@@ -48,6 +52,7 @@ def rules(tmp_path_factory):
     assert r.returncode == 0, r.stderr[-3000:]
     so = ctypes.CDLL(lib)
     so.rate_of.restype = ctypes.c_double
+    so.pre_max.restype = so.pre_top.restype = ctypes.c_longlong
 
     class Rules:
         @staticmethod
@@ -61,6 +66,14 @@ def rules(tmp_path_factory):
         @staticmethod
         def chunks(d, f64, law, rate, kind):
             return bool(so.chunks(d, int(f64), law, ctypes.c_double(rate), kind))
+
+        @staticmethod
+        def pre_max(d, f64, law, rate, kind):
+            return so.pre_max(d, int(f64), law, ctypes.c_double(rate), kind)
+
+        @staticmethod
+        def pre_top(d, f64):
+            return so.pre_top(d, int(f64))
 
         @staticmethod
         def ks_short(rate):
@@ -81,11 +94,11 @@ def test_a_problem_without_a_jump_law_has_no_rate(rules, d, f64):
     assert rules.rate(NONE, 5.0, 2.0, 100) == 0.0 and rules.rate(NORMAL, 5.0, 2.0, 100) == 0.1
     for rate in (0.002, 0.01, 0.05, 0.3):
         assert rules.chunk_len(d, NONE, rate) == 16
-        for kind in (PLAIN, STORE, REPLAY):
+        for kind in (COST, STORE, REPLAY):
             assert rules.chunks(d, f64, NONE, rate, kind) == rules.chunks(d, f64, NORMAL, 0.0, kind)
         assert rules.keeps(d, f64, NONE, rate) == rules.keeps(d, f64, NORMAL, 0.0)
     if d > 2:
-        assert not any(rules.chunks(d, f64, NONE, 0.01, kind) for kind in (PLAIN, STORE, REPLAY))
+        assert not any(rules.chunks(d, f64, NONE, 0.01, kind) for kind in (COST, STORE, REPLAY))
 
 
 @pytest.mark.parametrize("f64", [False, True])
@@ -94,7 +107,7 @@ def test_warp_wide_draws_need_a_one_jump_path(rules, f64):
     pairs than compiled (d = 5, 6 in the kernels of d = 8), have no one-jump path: the
     warp-wide form would cost and give nothing (KS d = 8, FP32, 0.02: store 1.52 -> 1.83 ms)."""
     rates = (0.002, 0.006, 0.012, 0.02, 0.05, 0.08)
-    kinds = (PLAIN, STORE, REPLAY)
+    kinds = (COST, STORE, REPLAY)
     for d in (3, 4, 7, 8):
         assert not any(rules.chunks(d, f64, KS, r, k) for r in rates for k in kinds)
         assert any(rules.chunks(d, f64, NORMAL, r, k) for r in rates for k in kinds)
@@ -111,17 +124,17 @@ CHUNKS = [
     (2, False, UNIFORM, STORE, 0.5, True),      # 3.23 -> 3.06
     (2, False, UNIFORM, STORE, 0.8, False),     # 3.87 -> 4.82
     (2, False, UNIFORM, PAIR, 0.8, False),      # 7.65 -> 9.41
-    (2, True, UNIFORM, PLAIN, 0.2, True),       # 3.22 -> 2.95
-    (2, True, UNIFORM, PLAIN, 0.4, False),      # 4.42 -> 4.71
+    (2, True, UNIFORM, COST, 0.2, True),       # 3.22 -> 2.95
+    (2, True, UNIFORM, COST, 0.4, False),      # 4.42 -> 4.71
     (1, True, NORMAL, STORE, 0.4, True),        # 4.64 -> 4.04
     (1, True, NORMAL, STORE, 0.8, False),       # 5.98 -> 6.81
     (2, True, KS, STORE, 0.0, False),           # 0.71 -> 0.79
     (2, True, KS, PAIR, 0.003, False),          # 1.17 -> 1.25
     (2, True, KS, STORE, 0.006, True),          # 1.04 -> 0.96
     (2, True, UNIFORM, STORE, 0.0, True),       # 0.81 -> 0.79
-    (1, False, NORMAL, PLAIN, 0.002, False),    # 0.945 -> 0.977
-    (1, False, NORMAL, PLAIN, 0.008, True),     # 1.20 -> 1.13
-    (2, False, UNIFORM, PLAIN, 0.0, True),      # 0.934 -> 0.894
+    (1, False, NORMAL, COST, 0.002, False),    # 0.945 -> 0.977
+    (1, False, NORMAL, COST, 0.008, True),     # 1.20 -> 1.13
+    (2, False, UNIFORM, COST, 0.0, True),      # 0.934 -> 0.894
     (2, False, UNIFORM, PAIR, 0.003, True),     # 1.417 -> 1.365 stored
 ]
 
@@ -164,5 +177,42 @@ def test_four_components_draw_warp_wide_where_that_gains(rules):
     for rate in (0.008, 0.012, 0.02, 0.03, 0.05):
         assert not rules.chunks(4, False, NORMAL, rate, STORE)
         assert rules.chunks(4, False, NORMAL, rate, REPLAY)
-    assert rules.chunks(4, False, NORMAL, 0.02, PLAIN)
-    assert not rules.chunks(4, False, NORMAL, 0.03, PLAIN) and not rules.chunks(4, False, NORMAL, 0.009, PLAIN)
+    assert rules.chunks(4, False, NORMAL, 0.02, COST)
+    assert not rules.chunks(4, False, NORMAL, 0.03, COST) and not rules.chunks(4, False, NORMAL, 0.009, COST)
+
+
+# (d, f64, kind, rate, M, pre-drawn): the sweep in the other form -> pre-drawn, us
+PRE = [
+    (1, False, STORE, 0.002, 2500, False),       # 52 -> 60
+    (1, False, STORE, 0.002, 5500, False),       # 53 -> 67
+    (1, False, COST, 0.002, 5500, True),         # 59 -> 50
+    (1, False, PAIR, 0.0005, 3000, False),       # 48 -> 74
+    (1, False, CKPT_PAIR, 0.007, 3000, True),    # 67 -> 60
+    (1, False, CKPT, 0.0005, 3000, True),        # 57 -> 50
+    (2, False, CKPT, 0.002, 4800, False),        # 55 -> 63
+    (2, False, STORE, 0.002, 4800, False),       # 59 -> 67
+    (2, False, COST, 0.02, 5500, True),
+    (1, False, STORE, 0.02, 1000, True),
+    (1, True, STORE, 0.002, 7500, True),         # 488 -> 378
+    (1, True, PAIR, 0.002, 7500, False),         # 610 -> 735
+    (2, True, PAIR, 0.002, 5500, False),         # 866 -> 1041
+    (2, True, STORE, 0.002, 5500, True),         # 627 -> 547
+    (2, True, PAIR, 0.2, 6000, True),            # 3189 -> 2890
+    (1, True, PAIR, 0.03, 7200, True),           # 955 -> 904
+]
+
+
+@pytest.mark.parametrize("d,f64,kind,rate,M,want", PRE)
+def test_pre_drawn_sweeps_where_they_are_faster(rules, d, f64, kind, rate, M, want):
+    assert (M <= rules.pre_max(d, f64, NORMAL, rate, kind)) == want
+
+
+@pytest.mark.parametrize("f64", [False, True])
+def test_pre_pass_buffers_cover_every_rate(rules, f64):
+    rates = (0.0, 0.001, 0.004, 0.005, 0.01, 0.03, 0.05, 0.3, 2.0)
+    for d in (1, 2):
+        for kind in (COST, CKPT, STORE, PAIR, CKPT_PAIR):
+            limits = [rules.pre_max(d, f64, NORMAL, r, kind) for r in rates]
+            assert f64 or limits == sorted(limits)
+            assert max(limits) <= rules.pre_top(d, f64)
+    assert rules.pre_max(4, f64, NORMAL, 0.1, COST) == rules.pre_top(4, f64) == 0
