@@ -40,6 +40,7 @@ struct KParams {
   uint32_t key0, key1, epoch;
   int d, npair, Nt, cubic, jump_law, jumps_on, has_dA, S, nblk;
   int kvel;                       // first component a jump moves (d/2 for Keilson-Storer, else 0)
+  int one_pairs;                  // npair, or 0 where no step takes the one-jump paths
   int64_t m_begin;                // global index of path 0 of this launch
   int64_t npart;                  // stride of the per-warp gradient partials (all launches)
   // Philox round keys (key0 + r W0, key1 + r W1 mod 2^32, r = 0..9), read by the forward
@@ -47,7 +48,6 @@ struct KParams {
   // block; last in the struct, so kernels that do not read them see the same layout
   uint32_t rk0[10], rk1[10];
   int chunk;                      // steps per chunk of the chunked forward sweep (4, 8 or 16)
-  int ks_one;                     // Keilson-Storer steps with one jump take the short path
 };
 
 // Device buffers of one launch (unused ones are null).

@@ -261,11 +261,12 @@ __host__ __device__ constexpr int seg_len() {
 // the additive laws for larger d (whose sweeps ran 1% slower with the law's branch).
 template <int D>
 constexpr bool ONE_JUMP_KS = D <= 2;
-// The step has exactly one jump and its slot words lie as compiled (the one-jump paths).
+// A step with jumps has exactly one, and the problem's steps take the one-jump paths (make_kparams;
+// a test of the law here beside that of the words cost the pre-drawn sweeps, whose steps are one
+// chain, 5%: d = 1 pair, M = 1000, N_t = 200, FP32, lambda dt = 0.07: 103 against 98 us).
 template <typename R, int D, int DU>
 __device__ __forceinline__ bool one_jump(const KParams<R, D, DU> &kp, uint32_t w0) {
-  return (kp.jump_law != JD_JUMP_KS || (ONE_JUMP_KS<D> && kp.ks_one)) && kp.npair == MainWords<D>::PD &&
-         (unsigned long long)w0 < kp.thr[1];
+  return kp.one_pairs == MainWords<D>::PD && (unsigned long long)w0 < kp.thr[1];
 }
 
 // The jump of a one-jump step (apply_jump; the additive map without its product by jgain = 1,
@@ -2572,7 +2573,7 @@ void make_kparams(const jd_problem *p, int64_t m_begin, int64_t mloc, KParams<R,
   kp.chunk = 4;
   if constexpr (fwd_chunked<D>())
     kp.chunk = fwd_chunk_len(jump_rate(q.jump_law, q.lambda, q.T, q.Nt), FwdChunk<R, D>::CH);
-  kp.ks_one = ks_one_jump(jump_rate(q.jump_law, q.lambda, q.T, q.Nt));
+  kp.one_pairs = one_jump_path(form_key(D, sizeof(R) == 8, q)) ? kp.npair : 0;
   kp.S = p->S;   // checkpoint spacing of the recompute plan (a power of two, 16 .. 64)
   kp.nblk = (int)ceil_div(mloc, TPB);
   kp.m_begin = q.m_offset + m_begin;   // global path index (a shard starts at m_offset)

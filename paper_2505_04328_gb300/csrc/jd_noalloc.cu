@@ -112,7 +112,7 @@ static void noalloc_kparams(const jd_problem_desc &q, KParams<R, D, DU> &kp) {
   kp.has_dA = 0;
   kp.S = seg_len<D>();
   kp.chunk = fwd_chunk_len(jump_rate(q.jump_law, q.lambda, q.T, q.Nt), FwdChunk<R, D>::CH);
-  kp.ks_one = 0;   // the law is not taken here
+  kp.one_pairs = one_jump_path(form_key(D, sizeof(R) == 8, q)) ? kp.npair : 0;
   kp.nblk = (int)ceil_div(q.M, TPB);
   kp.m_begin = q.m_offset;   // global index of the first path
   kp.npart = kp.nblk * (int64_t)(TPB / 32);

@@ -24,8 +24,8 @@ inline bool ks_one_jump(double rate) { return rate <= 0.5; }
 struct FormKey {
   int D;
   bool f64;
-  bool one_jump;   // steps with one jump take the short path (one_jump of the kernels): the
-                   // slot's words lie as compiled for D, and the law is additive for d > 2
+  bool one_jump;   // a step with one jump can take the short path: the slot's words lie as
+                   // compiled for D, and the law is additive for d > 2
   bool ks;         // Keilson-Storer law
   double rate;     // jump_rate
 };
@@ -45,6 +45,9 @@ inline int fwd_chunk_len(double rate, int most) {
 // What a launch runs: a forward sweep (cost, checkpoints, stored states; the last two also for a
 // pair of controls) or the replay of the recompute adjoint.
 enum SweepKind { SWEEP_COST, SWEEP_CKPT, SWEEP_STORE, SWEEP_STORE_PAIR, SWEEP_CKPT_PAIR, SWEEP_REPLAY };
+
+// Whether the steps with one jump take the short path.
+inline bool one_jump_path(const FormKey &f) { return f.one_jump && (!f.ks || ks_one_jump(f.rate)); }
 
 // d > 2: whether a one-jump step's slot draws are the whole warp's (coop_slot0_draws).  A lane
 // alone draws with its warp waiting; the warp-wide form costs the steps without jumps a
