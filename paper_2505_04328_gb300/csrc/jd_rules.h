@@ -28,11 +28,12 @@ struct FormKey {
                    // compiled for D, and the law is additive for d > 2
   bool ks;         // Keilson-Storer law
   double rate;     // jump_rate
+  int64_t M;       // paths
 };
 inline FormKey form_key(int D, bool f64, const jd_problem_desc &q) {
   const bool packed = (q.d + 1) / 2 == (D + 1) / 2;
   const bool ks = q.jump_law == JD_JUMP_KS;
-  return FormKey{D, f64, packed && (D <= 2 || !ks), ks, jump_rate(q.jump_law, q.lambda, q.T, q.Nt)};
+  return FormKey{D, f64, packed && (D <= 2 || !ks), ks, jump_rate(q.jump_law, q.lambda, q.T, q.Nt), q.M};
 }
 
 // Chunk length: the records hold a lane's jumps of a chunk but in rare chunks, and a pass of
@@ -61,19 +62,20 @@ inline bool one_jump_path(const FormKey &f) { return f.one_jump && (!f.ks || ks_
 //                            replay  0.57 -> 0.57   0.63 -> 0.61   0.81 -> 0.76   1.76 -> 1.57
 //   FP64 d = 8  M = 16,000   store   1.86 -> 1.86   2.20 -> 2.00   3.08 -> 2.50   5.63 -> 4.20
 //   FP64 d = 4               store   0.87 -> 0.88   1.02 -> 0.94   1.44 -> 1.20   2.53 -> 2.15
-// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)  The FP32
-// d = 4 cost and checkpoint sweeps gain between 0.01 and 0.03: cost 0.506 -> 0.499 ms at 0.01,
-// 0.571 -> 0.552 at 0.015, 0.632 -> 0.609 at 0.02, 0.735 -> 0.719 at 0.03 (M = 50,001: 0.161 ->
-// 0.161, 0.184 -> 0.181, 0.204 -> 0.203); its store sweep not for every size: 0.718 -> 0.700 at
-// 0.02, but 0.186 -> 0.190 at 0.01 and 0.271 -> 0.281 at 0.03 for M = 50,001.  Where no
-// step takes the one-jump path the form only costs: Keilson-Storer d = 8, FP32, M = 2^17, store
-// sweep 1.17 -> 1.33 ms at 0.01, 1.52 -> 1.83 at 0.02, cost 1.07 -> 1.17 and 1.47 -> 1.63.
+// (at 0.2 the warp-wide FP32 sweeps are slower again: d = 8 store 6.7 against 5.4.)  FP32 d = 4
+// gains only where the chip is full: replay at 0.02 0.173 -> 0.178 ms for M = 8000, 0.212 -> 0.207
+// at 20,000, 0.283 -> 0.261 at 40,000 (at 0.05 0.256 -> 0.285, 0.330 -> 0.332, 0.434 -> 0.398);
+// cost at 0.02 0.126 -> 0.135, 0.151 -> 0.157, 0.199 -> 0.197, 0.632 -> 0.609 at 200,003, and
+// between 0.01 and 0.03 only; its store sweep not for every size even there (0.718 -> 0.700 at
+// 200,003, but 0.271 -> 0.281 at 50,001 and 0.03).  Where no step takes the one-jump path the form
+// only costs: Keilson-Storer d = 8, FP32, M = 2^17, store sweep 1.17 -> 1.33 ms at 0.01, 1.52 ->
+// 1.83 at 0.02, cost 1.07 -> 1.17 and 1.47 -> 1.63.
 inline bool coop_slots(const FormKey &f, SweepKind kind) {
   if (!f.one_jump) return false;
   if (f.f64) return f.rate > 0.0005 && f.rate <= 0.1;
   if (f.D == 8) return f.rate > (kind == SWEEP_STORE ? 0.005 : 0.0015) && f.rate <= 0.08;
-  if (kind == SWEEP_REPLAY) return f.rate > 0.003 && f.rate <= 0.08;
-  return (kind == SWEEP_COST || kind == SWEEP_CKPT) && f.rate > 0.01 && f.rate <= 0.025;
+  if (kind == SWEEP_REPLAY) return f.M >= 152 * 128 && f.rate > 0.003 && f.rate <= 0.08;
+  return (kind == SWEEP_COST || kind == SWEEP_CKPT) && f.M >= 152 * 256 && f.rate > 0.01 && f.rate <= 0.025;
 }
 
 // d <= 2: whether a sweep takes its steps in chunks, by the jump rate per step.  The chunks'
@@ -95,14 +97,16 @@ inline bool coop_slots(const FormKey &f, SweepKind kind) {
 //               replay     1.05 -> 1.05  1.19 -> 1.18  1.41 -> 1.32  3.23 -> 2.87  6.76 -> 6.90  8.76 -> 9.30  9.49 -> 10.2
 //   FP64 KS     store      0.71 -> 0.79  0.84 -> 0.89  1.04 -> 0.96  2.68 -> 1.94  4.73 -> 4.42  5.79 -> 5.92  6.19 -> 6.48
 // (The FP32 replay of d = 2 also takes 0.73 -> 0.58 at 0.03, 3.95 -> 3.78 at 0.07 and 12.1 -> 13.4
-// at 0.2, M = 2^20; at 1.2 the FP32 store sweep of d = 2 takes 4.6 -> 6.3.)
+// at 0.2, M = 2^20: 5 blocks of it fit an SM in chunks, 6 step by step.  While all its blocks are
+// resident it is faster in chunks at every rate: at 0.2 0.744 -> 0.622 for M = 13,000, 1.37 -> 1.21
+// at 80,000, but 1.55 -> 2.11 at 110,000.  At 1.2 the FP32 store sweep of d = 2 takes 4.6 -> 6.3.)
 inline bool chunk_steps(const FormKey &f, SweepKind kind) {
   double lo = 0.0, hi = 0.5;
   if (f.f64) {
     if (f.D == 2) hi = 0.3;
     if (f.ks && kind != SWEEP_REPLAY) lo = 0.004;
   } else {
-    if (f.D == 2 && kind == SWEEP_REPLAY) hi = 0.08;
+    if (f.D == 2 && kind == SWEEP_REPLAY && f.M > 152 * 5 * 128) hi = 0.08;
     if (f.D == 1 && (kind == SWEEP_COST || kind == SWEEP_CKPT)) lo = 0.005;
   }
   return f.rate >= lo && f.rate <= hi;

@@ -13,6 +13,7 @@ COST, CKPT, STORE, PAIR, CKPT_PAIR, REPLAY = range(6)
 SRC = r"""
 #include "jd_rules.h"
 using namespace jd;
+static long long paths = 1 << 20;   // of the descriptors below
 static jd_problem_desc desc(int d, int law, double rate) {
   jd_problem_desc q{};
   q.d = d;
@@ -20,12 +21,14 @@ static jd_problem_desc desc(int d, int law, double rate) {
   q.Nt = 64;
   q.lambda = rate * 32.0;
   q.jump_law = (jd_jump_law)law;
+  q.M = paths;
   return q;
 }
 static FormKey key(int d, int f64, int law, double rate) {
   return form_key(d <= 2 ? d : d <= 4 ? 4 : 8, f64 != 0, desc(d, law, rate));
 }
 extern "C" {
+void set_paths(long long M) { paths = M; }
 double rate_of(int law, double lambda, double T, int Nt) { return jump_rate((jd_jump_law)law, lambda, T, Nt); }
 int chunk_len(int d, int law, double rate, int most) { return fwd_chunk_len(key(d, 0, law, rate).rate, most); }
 int chunks(int d, int f64, int law, double rate, int kind) {
@@ -64,7 +67,8 @@ def rules(tmp_path_factory):
             return so.chunk_len(d, law, ctypes.c_double(rate), most)
 
         @staticmethod
-        def chunks(d, f64, law, rate, kind):
+        def chunks(d, f64, law, rate, kind, M=1 << 20):
+            so.set_paths(ctypes.c_longlong(M))
             return bool(so.chunks(d, int(f64), law, ctypes.c_double(rate), kind))
 
         @staticmethod
@@ -216,3 +220,15 @@ def test_pre_pass_buffers_cover_every_rate(rules, f64):
             assert f64 or limits == sorted(limits)
             assert max(limits) <= rules.pre_top(d, f64)
     assert rules.pre_max(4, f64, NORMAL, 0.1, COST) == rules.pre_top(4, f64) == 0
+
+
+def test_forms_by_the_number_of_paths(rules):
+    """FP32 d = 2 replay at high rates: in chunks while its blocks are resident (M = 80,000 1.37
+    -> 1.21 ms at 0.2, 110,000 1.55 -> 2.11).  FP32 d = 4 warp-wide draws: from a full chip on
+    (replay at 0.05, M = 8000 0.256 -> 0.285, 40,000 0.434 -> 0.398)."""
+    for law in (UNIFORM, KS):
+        assert rules.chunks(2, False, law, 0.2, REPLAY, M=13000) and rules.chunks(2, False, law, 0.2, REPLAY, M=80000)
+        assert not rules.chunks(2, False, law, 0.2, REPLAY, M=110000)
+    for kind, M in ((REPLAY, 8000), (COST, 8000), (CKPT, 20000)):
+        assert not rules.chunks(4, False, NORMAL, 0.02, kind, M=M)
+        assert rules.chunks(4, False, NORMAL, 0.02, kind, M=80000)
