@@ -71,6 +71,7 @@ struct FbParams {
   const R *z0;              // interacting particles: initial states [2][S] (on the ellipse)
   int gauss, ellipse, N, Nt;   // N: particles per ring, 0 = independent paths
   int S;                    // lanes (path indices) per ring: particle i of ring r is lane S r + i
+  int one_slot;             // a step with one jump takes its slot's draws in straight code (fb_one_slot)
   int64_t mloc;
 };
 
@@ -474,12 +475,12 @@ fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant
       const uint32_t w0 = main_draws<true>(kp, k, mg, zs);   // round keys of the parameter block
       int n = 0;
       FbPlan<R> P;
-      // a step with one jump takes its slot's draws in straight code, any other jump step the
-      // plan's loops
+      // a step with one jump takes its slot's draws in straight code where that pays
+      // (fb_one_slot; FP32 only), any other jump step the plan's loops
       bool one = false, log = false;
       R th1 = R(1), xih1[2] = {R(0), R(0)}, z1[2] = {R(0), R(0)};
       if (has_jump(kp, w0)) {
-        one = (unsigned long long)w0 < kp.thr[1];
+        one = sizeof(R) == 4 && fp.one_slot && (unsigned long long)w0 < kp.thr[1];
         if (one) {
           n = 1;
           th1 = slot_draws_at<true>(kp, k, mg, 0, xih1, z1);
@@ -1006,6 +1007,8 @@ void fb_make_params(const ::jd_problem *p, const jd_feedback_desc &fb, FbParams<
   fp.iav2 = (R)(fb.track == JD_TRACK_ELLIPSE || fb.particles ? 1.0 / (fb.av * fb.av) : 0.0);
   fp.N = fb.particles;
   fp.S = fb.particles ? ring_lanes(fb.particles) : 0;
+  fp.one_slot = fb_one_slot(sizeof(R) == 8, ring_kind(fb.particles),
+                            jump_rate(p->desc.jump_law, p->desc.lambda, p->desc.T, p->desc.Nt));
   fp.omega = (R)fb.omega;
   fp.z0 = static_cast<const R *>(p->fb_z0);   // the ring's initial states (fb_upload_ring)
   fp.Nt = p->desc.Nt;

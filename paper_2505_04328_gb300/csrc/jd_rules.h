@@ -181,4 +181,20 @@ inline bool theta_keeps(const FormKey &f) {
   return f.rate > 0.0 && f.rate <= (f.f64 ? 0.16 : f.ks ? 0.11 : 0.12);
 }
 
+// Feedback forward sweep: whether a step with one jump takes its slot's draws in straight code
+// beside the plan's loops of the other jump steps.  At high rates a warp runs both at nearly every
+// step, sooner where a ring's lanes wait for one another (ring_kind 2 and 3); in FP64 the loops
+// cost no more than the straight code at any rate.  Forward without stored states, N_t = 60,
+// loops -> straight, in us (FP32 M = 2^18, FP64 2^15):
+//   lambda dt                   0.02          0.1           0.15          0.2           0.3           1
+//   FP32 4 x 4                  396 -> 282    641 -> 487    704 -> 604    765 -> 720    880 -> 927    1439 -> 1578
+//        10 x 10                522 -> 417    820 -> 675    897 -> 800    975 -> 934    1122 -> 1173  1832 -> 1970
+//        16 x 16                813 -> 728    1205 -> 1094  1318 -> 1246  1428 -> 1396  1641 -> 1684  2677 -> 2785
+//        4 x 4, rings of 200    491 -> 334    686 -> 648    762 -> 801    828 -> 890    939 -> 1034   1514 -> 1652
+//        16 x 16, rings of 200  999 -> 826    1392 -> 1351  1537 -> 1565  1650 -> 1722  1855 -> 1951  2913 -> 3045
+//   FP64 10 x 10                4517 -> 4506  6449 -> 6537  7090 -> 7238  7563 -> 7817  8769 -> 9144  14026 -> 14455
+inline bool fb_one_slot(bool f64, int ring_kind, double rate) {
+  return !f64 && rate <= (ring_kind <= 1 ? 0.25 : 0.13);
+}
+
 }  // namespace jd

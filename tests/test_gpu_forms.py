@@ -89,3 +89,24 @@ def test_pre_drawn_sweeps_equal_the_others(law, prec, Nt, lamdt):
         part, npart = _launches(lambda: jp.cost_units(u))
         assert np.array_equal(grads[1:], jp.gradient_units(u))
     assert npart == n + PRE_EXTRA and np.array_equal(whole[1:], part)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+@pytest.mark.parametrize("particles,lamdt", [(0, 0.24), (0, 0.27), (200, 0.12), (200, 0.14), (200, 1.5)])
+def test_feedback_across_the_straight_code_limit(particles, lamdt, prec):
+    """Either side of the rate that decides on a one-jump step's draws, against the oracle.
+    FP32: 20 steps of 2.5 sub-steps with 4 roundings each of 2^-24 are 1.2e-5 of a path's value
+    at worst, ten times that for the adjoint's weights."""
+    Nt = 20
+    M = oracle.ring_lanes(particles) * 2 if particles else 600
+    p, fb = workloads.feedback_coupled(M=M, Nt=Nt, particles=particles) if particles else \
+        workloads.feedback_centering(M=M, Nt=Nt)
+    p = p.replace(lam=lamdt * Nt / p.T)
+    mu = workloads.random_mu(p, fb, seed=8, scale=0.5)
+    Jo, go = (oracle.fb_coupled_gradient if particles else oracle.fb_gradient)(p, fb, mu)[:2]
+    with JdProblem(p, prec=prec) as jp:
+        J, g = jp.fb_gradient(fb, mu)
+        assert jp.fb_cost(fb, mu) == J
+    tol_j, tol_g = (1e-13, 1e-12) if prec == "fp64" else (1.2e-5, 1.2e-4)
+    assert abs(J - Jo) <= tol_j * abs(Jo)
+    assert np.linalg.norm(g - go) <= tol_g * np.linalg.norm(go)
