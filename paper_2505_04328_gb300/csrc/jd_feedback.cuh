@@ -412,20 +412,37 @@ __device__ __forceinline__ double fb_block_sum(Pair<R> v, Pair<R> *red) {
   return out;
 }
 
-// Resident blocks per SM asked of the compiler (its own choice took 98 registers forward and
-// 230 in the adjoint with the jump log): FP32 10 x 10 forward 3 blocks of 80 registers 2.56 ms,
-// unbounded 3.64 (M = 2^20, N_t = 100); adjoint 2 blocks of 128 4.30, unbounded 5.35, 3 of 80
-// 4.90.
-template <typename R, int NX, int NV>
+// Resident blocks per SM asked of the compiler.  FP32, its own choice -> bounded, forward with
+// stored states and adjoint, in us (M = 2^18, N_t = 60, lambda dt = 0.018):
+//   4 x 4    forward 304 -> 300 (3 blocks)   adjoint 374 -> 351 (3)
+//   10 x 10  forward 458 -> 429 (3)          adjoint 705 -> 702 (2)
+//   16 x 16  forward 724 -> 735 (2)          adjoint 1336 -> 1236 (2; 12 to 56 bytes spilled)
+//   rings of 200: 10 x 10 forward 596 -> 494, 16 x 16 adjoint 1824 -> 1453
+// FP64: one block fills the pipe, so the time is blocks per SM, rounded up to whole rounds, and a
+// second resident block only makes the rounds coarser; but the lanes of a block's ring wait for
+// one another, and a second block fills that.  Two blocks asked -> one, forward, in ms (N_t = 40,
+// lambda dt = 0.018, M = 2^17; 100,096, which is 2.6 rounds of one block):
+//   10 x 10  11.3 -> 11.4; 11.0 -> 8.6     rings of 200  9.5 -> 10.6; 9.3 -> 8.0
+//   16 x 16  18.7 -> 19.0; 18.3 -> 14.4    rings of 200  16.4 -> 17.3; 15.8 -> 13.0
+// so one block but for the 10 x 10 rings, whose second block earns more.  The adjoint takes one.
+template <typename R, int NX, int NV, int RING>
 constexpr int fb_fwd_blocks() {
-  return sizeof(R) == 8 || NX * NV > 100 ? 2 : 3;
+  if (sizeof(R) == 8) return RING >= 2 && NX * NV <= 100 ? 2 : 1;
+  return NX * NV > 100 ? 2 : 3;
 }
 template <typename R, int NX, int NV>
 constexpr int fb_adj_blocks() {
   return sizeof(R) == 8 ? 1 : NX * NV <= 16 ? 3 : 2;
 }
+// The FP64 4 x 4 forward of independent paths needs few registers (114), so two of its blocks
+// would share an SM: dynamic shared memory that it does not use keeps the second out.  Cost at
+// M = 100,096 5.17 -> 4.00 ms, at 2^17 5.24 -> 5.26.
+template <typename R, int NX, int NV, int RING>
+constexpr size_t fb_fwd_pad() {
+  return sizeof(R) == 8 && NX * NV <= 16 && RING <= 1 ? 116 * 1024 : 0;
+}
 template <typename R, int NX, int NV, bool STORE, int RING>
-__global__ void __launch_bounds__(FB_TPB, fb_fwd_blocks<R, NX, NV>())
+__global__ void __launch_bounds__(FB_TPB, fb_fwd_blocks<R, NX, NV, RING>())
 fb_fwd_kernel(const __grid_constant__ KParams<R, 2, 1> kp, const __grid_constant__ FbParams<R> fp,
               const R *__restrict__ mu, const R *__restrict__ xd, R *__restrict__ traj,
               uint32_t *__restrict__ flags, JLog<R, 2> jl, int *__restrict__ jcnt, double *__restrict__ partC) {
@@ -1055,7 +1072,10 @@ JLog<R, 2> fb_log(const FbBufs &b, int64_t mloc) {
 template <typename R, int NX, int NV, bool STORE, int RING>
 cudaError_t fb_fwd_ring(const KParams<R, 2, 1> &kp, const FbParams<R> &fp, const R *mu, const R *xd, const FbBufs &b,
                         unsigned grid, cudaStream_t s) {
-  return fb_launch(fb_fwd_kernel<R, NX, NV, STORE, RING>, RING, fp.S, grid, 0, s, kp, fp, mu, xd,
+  constexpr size_t pad = fb_fwd_pad<R, NX, NV, RING>();
+  const cudaError_t e = ensure_dyn_smem((const void *)fb_fwd_kernel<R, NX, NV, STORE, RING>, pad);
+  if (e != cudaSuccess) return e;
+  return fb_launch(fb_fwd_kernel<R, NX, NV, STORE, RING>, RING, fp.S, grid, pad, s, kp, fp, mu, xd,
                    STORE ? static_cast<R *>(b.traj) : nullptr, STORE ? b.flags : nullptr, fb_log<R>(b, fp.mloc),
                    STORE ? b.jcnt : nullptr, b.partC);
 }

@@ -110,3 +110,20 @@ def test_feedback_across_the_straight_code_limit(particles, lamdt, prec):
     tol_j, tol_g = (1e-13, 1e-12) if prec == "fp64" else (1.2e-5, 1.2e-4)
     assert abs(J - Jo) <= tol_j * abs(Jo)
     assert np.linalg.norm(g - go) <= tol_g * np.linalg.norm(go)
+
+
+@pytest.mark.parametrize("nx", [4, 10, 16])
+@pytest.mark.parametrize("particles", [0, 20, 200])
+def test_feedback_fp64_sizes_and_rings(nx, particles):
+    """Every FP64 forward's own residency: costs and gradients against the oracle."""
+    Nt = 12
+    M = 512 if particles else 700
+    p, fb = workloads.feedback_coupled(M=M, Nt=Nt, particles=particles) if particles else \
+        workloads.feedback_centering(M=M, Nt=Nt)
+    p, fb = p.replace(lam=3.0), fb.replace(nx=nx, nv=nx)
+    mu = workloads.random_mu(p, fb, seed=8, scale=0.5)
+    Jo, go = (oracle.fb_coupled_gradient if particles else oracle.fb_gradient)(p, fb, mu)[:2]
+    with JdProblem(p, prec="fp64") as jp:
+        J, g = jp.fb_gradient(fb, mu)
+        assert jp.fb_cost(fb, mu) == J
+    assert abs(J - Jo) <= 1e-13 * abs(Jo) and np.linalg.norm(g - go) <= 1e-12 * np.linalg.norm(go)
