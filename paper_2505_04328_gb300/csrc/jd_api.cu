@@ -2010,8 +2010,9 @@ static jd_status fb_upload_ring(jd_problem *p, const jd_feedback_desc &fb) {
 }
 
 // Buffers of the feedback sweeps for padded size LP (the gradient also needs the states,
-// the flags and the gradient partials); raises the stack limit for the jump routines.
-static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad) {
+// the flags and the gradient partials; the exact adjoint's sweeps also the jump log, where there is
+// room); raises the stack limit for the jump routines.
+static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad, bool log) {
   const int LP = ops->NX * ops->NV, Nt = p->desc.Nt;
   const int64_t M = p->desc.M, nblk = ceil_div(M, FB_TPB);
   const size_t es = elem_size(p);
@@ -2039,7 +2040,7 @@ static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad) {
     s = dev_alloc(p, (void **)&p->fb_partG, (size_t)fb_groups(nwarp) * Nt * LP * 8, "feedback group partials");
   if (!s && !p->fb_z0) s = dev_alloc(p, &p->fb_z0, (size_t)2 * RING_MAX * es, "ring initial states");
   if (s) return s;
-  if (grad && p->fb_log_state == 0) {   // last, and only where there is room
+  if (log && p->fb_log_state == 0) {   // last, and only where there is room
     const int cap = log_capacity(p->desc);
     const size_t nk = (size_t)cap * M * 2 * es, nb = 2 * nk + (size_t)M * 8;
     p->fb_log_state = -1;
@@ -2084,7 +2085,8 @@ static jd_status fb_run(jd_problem *p, const jd_feedback_desc *fb, const double 
   const int Nt = p->desc.Nt;
   const size_t L = (size_t)fb->nx * fb->nv;
   s = set_device(p);
-  if (!s) s = fb_ensure(p, ops, grad_out != nullptr || store);
+  const bool exact = fb->adjoint == JD_FB_EXACT;   // the surrogate adjoint reads no log
+  if (!s) s = fb_ensure(p, ops, grad_out != nullptr || store, exact && (grad_out != nullptr || store));
   if (s) return s;
   const double *mud = mu;
   if (ms == JD_MEM_HOST) {

@@ -1,0 +1,38 @@
+"""The feedback sweep's optional jump log: when it is allocated, how large, and what it leaves
+to others.  Results never depend on it."""
+import numpy as np
+import pytest
+
+import workloads
+from paper_2505_04328_gb300 import JdProblem, build
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def _built():
+    build()
+
+
+def _problem(M=3000, Nt=45, **kw):
+    p, fb = workloads.feedback_centering(M=M, Nt=Nt)
+    p = p.replace(**kw)
+    return p, fb, workloads.random_mu(p, fb, seed=5, scale=0.4)
+
+
+def _bytes(jp):
+    return jp.info()["device_bytes"]
+
+
+def test_surrogate_adjoint_takes_no_log():
+    """Its sweeps neither write nor read the log."""
+    p, fb, mu = _problem()
+    with JdProblem(p) as jp:
+        jp.fb_gradient(fb.replace(adjoint=workloads.FB_SURROGATE, sur_rate=0.05), mu)
+        without = _bytes(jp)
+        J, g = jp.fb_gradient(fb, mu)
+        assert _bytes(jp) > without
+    with JdProblem(p, mem_budget=without + 8) as jp:
+        J0, g0 = jp.fb_gradient(fb, mu)
+        assert _bytes(jp) == without
+    assert J == J0 and np.array_equal(g, g0)
