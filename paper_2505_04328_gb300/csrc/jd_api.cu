@@ -501,15 +501,20 @@ static void drop_fb_log(jd_problem *p) {
 // Device bytes in use besides the droppable log.
 static size_t held_bytes(const jd_problem *p) { return p->bytes - p->fb_log_bytes; }
 
+// The one allocation of a problem's device memory, as free_dev frees it.
+static cudaError_t raw_alloc(jd_problem *p, void **ptr, size_t bytes) {
+  return p->async_alloc ? cudaMallocAsync(ptr, bytes, p->stream) : cudaMalloc(ptr, bytes);
+}
+
 static jd_status dev_alloc(jd_problem *p, void **ptr, size_t bytes, const char *what) {
   if (p->bytes + bytes > p->budget && p->fb_log_bytes) drop_fb_log(p);
   if (p->bytes + bytes > p->budget)
     return fail(JD_ERR_OOM, std::string("memory budget exceeded allocating ") + what);
-  cudaError_t e = p->async_alloc ? cudaMallocAsync(ptr, bytes, p->stream) : cudaMalloc(ptr, bytes);
+  cudaError_t e = raw_alloc(p, ptr, bytes);
   if (e != cudaSuccess && p->fb_log_bytes) {
     cudaGetLastError();
     drop_fb_log(p);
-    e = p->async_alloc ? cudaMallocAsync(ptr, bytes, p->stream) : cudaMalloc(ptr, bytes);
+    e = raw_alloc(p, ptr, bytes);
   }
   if (e != cudaSuccess) {
     cudaGetLastError();
@@ -2045,8 +2050,8 @@ static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad, bool log)
     const size_t nk = (size_t)cap * M * 2 * es, nb = 2 * nk + (size_t)M * 8;
     p->fb_log_state = -1;
     if (cap > 0 && p->bytes + nb <= p->budget) {
-      if (cudaMalloc(&p->fb_log_kt, nk) == cudaSuccess && cudaMalloc(&p->fb_log_y, nk) == cudaSuccess &&
-          cudaMalloc((void **)&p->fb_jcnt, (size_t)M * 8) == cudaSuccess) {
+      if (raw_alloc(p, &p->fb_log_kt, nk) == cudaSuccess && raw_alloc(p, &p->fb_log_y, nk) == cudaSuccess &&
+          raw_alloc(p, (void **)&p->fb_jcnt, (size_t)M * 8) == cudaSuccess) {
         p->fb_log_bytes = nb;
         p->bytes += nb;
         p->fb_log_cap = cap;
