@@ -2046,7 +2046,7 @@ static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad, bool log)
   if (!s && !p->fb_z0) s = dev_alloc(p, &p->fb_z0, (size_t)2 * RING_MAX * es, "ring initial states");
   if (s) return s;
   if (log && p->fb_log_state == 0) {   // last, and only where there is room
-    const int cap = log_capacity(p->desc);
+    const int cap = fb_log_capacity(p->desc);
     const size_t nk = (size_t)cap * M * 2 * es, nb = 2 * nk + (size_t)M * 8;
     p->fb_log_state = -1;
     if (cap > 0 && p->bytes + nb <= p->budget) {

@@ -2,6 +2,8 @@
 // jump law and jump rate.  Plain C++ without CUDA, so that any host can check them.
 #pragma once
 
+#include <algorithm>
+#include <cmath>
 #include <cstdint>
 
 #include "jd.h"
@@ -195,6 +197,24 @@ inline bool theta_keeps(const FormKey &f) {
 //   FP64 10 x 10                4517 -> 4506  6449 -> 6537  7090 -> 7238  7563 -> 7817  8769 -> 9144  14026 -> 14455
 inline bool fb_one_slot(bool f64, int ring_kind, double rate) {
   return !f64 && rate <= (ring_kind <= 1 ? 0.25 : 0.13);
+}
+
+// Feedback jump log: records per path (at most 1024; 0: no jumps).  The expected records and a
+// wide Poisson margin; in FP32 only of the steps that are logged: a path's log closes at its first
+// step with three jumps (probability p3 per step) and a logged step has one or two records, so at
+// lambda dt = 0.5 and N_t = 1000 the log holds 69 steps on average and 1000 steps' records would
+// be mostly never written.  Four times the mean number of logged steps covers 98% of the paths.
+inline int fb_log_capacity(const jd_problem_desc &q) {
+  const double r = jump_rate(q.jump_law, q.lambda, q.T, q.Nt);
+  if (!(r > 0.0)) return 0;
+  double steps = q.Nt, most = 1024.0;
+  if (q.prec == JD_FP32) {
+    const double p3 = r < 0.05 ? r * r * r / 6.0 * (1.0 - 0.75 * r) : 1.0 - std::exp(-r) * (1.0 + r + 0.5 * r * r);
+    if (p3 * q.Nt > 1e-3) steps = std::min(steps, std::ceil(4.0 * (1.0 - std::pow(1.0 - p3, q.Nt)) / p3));
+    most = std::min(most, 2.0 * steps);
+  }
+  const double mean = r * steps;
+  return (int)std::min(most, std::ceil(mean + 6.0 * std::sqrt(mean) + 8.0));
 }
 
 }  // namespace jd

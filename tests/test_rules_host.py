@@ -39,6 +39,15 @@ long long pre_max(int d, int f64, int law, double rate, int kind) {
 }
 long long pre_top(int d, int f64) { return pre_top_paths(d, f64 != 0); }
 int one_slot(int f64, int ring, double rate) { return fb_one_slot(f64 != 0, ring, rate); }
+int log_capacity(int f64, int law, double rate, int Nt) {
+  jd_problem_desc q{};
+  q.T = 1.0;
+  q.Nt = Nt;
+  q.lambda = rate * Nt;
+  q.jump_law = (jd_jump_law)law;
+  q.prec = f64 ? JD_FP64 : JD_FP32;
+  return fb_log_capacity(q);
+}
 int ks_short(double rate) { return ks_one_jump(rate); }
 int keeps(int d, int f64, int law, double rate) { return theta_keeps(key(d, f64, law, rate)); }
 }
@@ -83,6 +92,10 @@ def rules(tmp_path_factory):
         @staticmethod
         def one_slot(f64, ring, rate):
             return bool(so.one_slot(int(f64), ring, ctypes.c_double(rate)))
+
+        @staticmethod
+        def log_capacity(f64, law, rate, Nt):
+            return so.log_capacity(int(f64), law, ctypes.c_double(rate), Nt)
 
         @staticmethod
         def ks_short(rate):
@@ -247,3 +260,18 @@ def test_feedback_straight_one_jump_code_where_it_is_faster(rules):
     for ring in (2, 3):
         assert rules.one_slot(False, ring, 0.1) and not rules.one_slot(False, ring, 0.15)
     assert not any(rules.one_slot(True, ring, r) for ring in range(4) for r in (0.0, 0.02, 0.1, 1.0))
+
+
+def test_feedback_log_capacity(rules):
+    """The centering problem's 18 records as before; in FP32 no more than the steps before the
+    first one with three jumps need (642 records at 0.5 and 1000 steps before); at least one."""
+    for f64 in (False, True):
+        assert rules.log_capacity(f64, KS, 0.0178, 100) == 18
+        assert rules.log_capacity(f64, KS, 0.0, 100) == 0 and rules.log_capacity(f64, NONE, 0.1, 100) == 0
+    assert rules.log_capacity(True, KS, 0.5, 1000) == 643
+    assert 69 * 0.5 * 2 < rules.log_capacity(False, KS, 0.5, 1000) < 230
+    # p3 = 0.9938: 1.0063 logged steps on average, four times that rounds up to 5, two records each
+    assert rules.log_capacity(False, KS, 9.0, 45) == 10
+    rates = (1e-7, 1e-4, 0.01, 0.0499, 0.0501, 0.2)
+    caps = [rules.log_capacity(False, KS, r, 100) for r in rates]
+    assert caps == sorted(caps) and caps == [rules.log_capacity(True, KS, r, 100) for r in rates]
