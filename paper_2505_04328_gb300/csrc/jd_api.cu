@@ -1864,6 +1864,10 @@ jd_status jd_problem_update(jd_problem *p, const jd_problem_desc *desc) {
   p->desc.u_max = q.u_max;
   p->desc.seed = q.seed;
   p->desc.epoch = q.epoch;
+  if (fb_log_capacity(p->desc) > p->fb_log_cap) {   // more jumps than the log was made for, or none yet
+    drop_fb_log(p);
+    p->fb_log_state = 0;   // the next gradient under feedback tries again
+  }
   if (new_target) {
     const cudaError_t e = upload_target(p);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy target");

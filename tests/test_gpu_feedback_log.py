@@ -36,3 +36,25 @@ def test_surrogate_adjoint_takes_no_log():
         J0, g0 = jp.fb_gradient(fb, mu)
         assert _bytes(jp) == without
     assert J == J0 and np.array_equal(g, g0)
+
+
+@pytest.mark.parametrize("prec", ["fp32", "fp64"])
+def test_log_follows_an_update(prec):
+    """A problem made without jumps gets its log when an update brings them, one made with few a
+    larger log when they become many; the results are a fresh problem's."""
+    none, fb, mu = _problem(lam=0.0)
+    few, many = none.replace(lam=2.0), none.replace(lam=8.0)
+    with JdProblem(none, prec=prec) as jp:
+        jp.fb_gradient(fb, mu)
+        sizes, out = [_bytes(jp)], []
+        for p in (few, many, few):
+            jp.update(p)
+            out.append(jp.fb_gradient(fb, mu))
+            sizes.append(_bytes(jp))
+    assert sizes[0] < sizes[1] < sizes[2] == sizes[3]
+    for p, (J, g) in zip((few, many, few), out):
+        with JdProblem(p, prec=prec) as jp:
+            J0, g0 = jp.fb_gradient(fb, mu)
+            if p is many:
+                assert _bytes(jp) == sizes[2]
+        assert J == J0 and np.array_equal(g, g0)
