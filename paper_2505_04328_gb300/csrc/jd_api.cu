@@ -488,7 +488,8 @@ static void free_dev(const jd_problem *p, T *&ptr) {
 }
 
 // The feedback sweep's jump log is optional (without it the adjoint regenerates the jump
-// steps): an allocation that finds no room takes its memory.
+// steps): an allocation of the problem that finds no room takes its memory, and it is made only
+// where the device keeps three times its size for others.
 static void drop_fb_log(jd_problem *p) {
   free_dev(p, p->fb_log_kt);
   free_dev(p, p->fb_log_y);
@@ -496,7 +497,7 @@ static void drop_fb_log(jd_problem *p) {
   p->bytes -= p->fb_log_bytes;
   p->fb_log_bytes = 0;
   p->fb_log_cap = 0;
-  p->fb_log_state = -1;
+  p->fb_log_state = 0;   // tried again where the budget has room
 }
 // Device bytes in use besides the droppable log.
 static size_t held_bytes(const jd_problem *p) { return p->bytes - p->fb_log_bytes; }
@@ -1864,10 +1865,8 @@ jd_status jd_problem_update(jd_problem *p, const jd_problem_desc *desc) {
   p->desc.u_max = q.u_max;
   p->desc.seed = q.seed;
   p->desc.epoch = q.epoch;
-  if (fb_log_capacity(p->desc) > p->fb_log_cap) {   // more jumps than the log was made for, or none yet
-    drop_fb_log(p);
-    p->fb_log_state = 0;   // the next gradient under feedback tries again
-  }
+  // more jumps than the log was made for, or no log yet: the next gradient under feedback tries
+  if (fb_log_capacity(p->desc) > p->fb_log_cap) drop_fb_log(p);
   if (new_target) {
     const cudaError_t e = upload_target(p);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMemcpy target");
@@ -2052,9 +2051,10 @@ static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad, bool log)
   if (log && p->fb_log_state == 0) {   // last, and only where there is room
     const int cap = fb_log_capacity(p->desc);
     const size_t nk = (size_t)cap * M * 2 * es, nb = 2 * nk + (size_t)M * 8;
-    p->fb_log_state = -1;
-    if (cap > 0 && p->bytes + nb <= p->budget) {
-      if (raw_alloc(p, &p->fb_log_kt, nk) == cudaSuccess && raw_alloc(p, &p->fb_log_y, nk) == cudaSuccess &&
+    size_t free_b = 0, total = 0;
+    if (cap > 0 && p->bytes + nb <= p->budget && cudaMemGetInfo(&free_b, &total) == cudaSuccess) {
+      if (fb_log_fits(nb, free_b) && raw_alloc(p, &p->fb_log_kt, nk) == cudaSuccess &&
+          raw_alloc(p, &p->fb_log_y, nk) == cudaSuccess &&
           raw_alloc(p, (void **)&p->fb_jcnt, (size_t)M * 8) == cudaSuccess) {
         p->fb_log_bytes = nb;
         p->bytes += nb;
@@ -2063,6 +2063,7 @@ static jd_status fb_ensure(jd_problem *p, const FbOps *ops, bool grad, bool log)
       } else {
         cudaGetLastError();
         drop_fb_log(p);
+        p->fb_log_state = -1;   // not before an update asks for another size
       }
     }
   }

@@ -277,7 +277,7 @@ struct jd_problem {
   double *fb_mu64 = nullptr, *fb_grad = nullptr, *fb_partC = nullptr, *fb_partG = nullptr;
   void *fb_partW = nullptr;
   // post-jump states of the feedback sweep for its adjoint, kept while the budget has room
-  // (dev_alloc drops them first); fb_log_state: 0 not tried, 1 there, -1 without
+  // (dev_alloc drops them first); fb_log_state: 0 to be tried, 1 there, -1 the device has no room
   void *fb_log_kt = nullptr, *fb_log_y = nullptr;
   int *fb_jcnt = nullptr;
   int fb_log_cap = 0, fb_log_state = 0;

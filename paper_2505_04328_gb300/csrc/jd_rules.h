@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <cmath>
+#include <cstddef>
 #include <cstdint>
 
 #include "jd.h"
@@ -216,5 +217,10 @@ inline int fb_log_capacity(const jd_problem_desc &q) {
   const double mean = r * steps;
   return (int)std::min(most, std::ceil(mean + 6.0 * std::sqrt(mean) + 8.0));
 }
+
+// Whether the device has room for a feedback jump log of that many bytes: another problem or
+// another library on the device cannot ask for its memory back, so it takes a quarter of what is
+// free at most.
+inline bool fb_log_fits(size_t bytes, size_t free_bytes) { return bytes <= free_bytes / 4; }
 
 }  // namespace jd

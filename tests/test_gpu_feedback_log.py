@@ -58,3 +58,26 @@ def test_log_follows_an_update(prec):
             if p is many:
                 assert _bytes(jp) == sizes[2]
         assert J == J0 and np.array_equal(g, g0)
+
+
+def test_a_smaller_log_after_one_that_gave_way():
+    """A log that made room for another allocation is tried again in the size of the present
+    jumps: with fewer of them it fits beside."""
+    p, fb, mu = _problem(M=4096, Nt=40, lam=8.0)
+    fewer, u = p.replace(lam=0.5), np.zeros((p.Nt, 1))
+    with JdProblem(p, mode="recompute") as jp:
+        jp.fb_gradient(fb, mu)
+        jp.gradient(u)
+        both = _bytes(jp)
+    with JdProblem(fewer) as jp:
+        J, g = jp.fb_gradient(fb, mu)
+    with JdProblem(p, mode="recompute", mem_budget=both - 8) as jp:
+        jp.fb_gradient(fb, mu)
+        jp.gradient(u)                      # takes the log's memory
+        dropped = _bytes(jp)
+        jp.fb_gradient(fb, mu)
+        assert _bytes(jp) == dropped < both - 8
+        jp.update(fewer)
+        J1, g1 = jp.fb_gradient(fb, mu)
+        assert dropped < _bytes(jp) <= both - 8
+    assert J1 == J and np.array_equal(g1, g)

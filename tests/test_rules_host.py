@@ -48,6 +48,7 @@ int log_capacity(int f64, int law, double rate, int Nt) {
   q.prec = f64 ? JD_FP64 : JD_FP32;
   return fb_log_capacity(q);
 }
+int log_fits(long long bytes, long long free_bytes) { return fb_log_fits((size_t)bytes, (size_t)free_bytes); }
 int ks_short(double rate) { return ks_one_jump(rate); }
 int keeps(int d, int f64, int law, double rate) { return theta_keeps(key(d, f64, law, rate)); }
 }
@@ -96,6 +97,10 @@ def rules(tmp_path_factory):
         @staticmethod
         def log_capacity(f64, law, rate, Nt):
             return so.log_capacity(int(f64), law, ctypes.c_double(rate), Nt)
+
+        @staticmethod
+        def log_fits(need, free):
+            return bool(so.log_fits(ctypes.c_longlong(need), ctypes.c_longlong(free)))
 
         @staticmethod
         def ks_short(rate):
@@ -275,3 +280,10 @@ def test_feedback_log_capacity(rules):
     rates = (1e-7, 1e-4, 0.01, 0.0499, 0.0501, 0.2)
     caps = [rules.log_capacity(False, KS, r, 100) for r in rates]
     assert caps == sorted(caps) and caps == [rules.log_capacity(True, KS, r, 100) for r in rates]
+
+
+def test_feedback_log_leaves_room_for_others(rules):
+    """The default memory budget is half of what is free; a log of that size would leave a second
+    problem with the same default half of the rest."""
+    assert rules.log_fits(1 << 30, 4 << 30) and not rules.log_fits((1 << 30) + 1, 4 << 30)
+    assert not rules.log_fits(1, 3) and rules.log_fits(70 << 30, 283 << 30)
