@@ -81,8 +81,12 @@ static cudaError_t op32_adj(const jd_problem *p, int variant, bool theta, int64_
   return cudaGetLastError();
 }
 
+// The kernels' own frames (432 bytes at most; adj32_jump_substeps, their only call, keeps its
+// values in registers) and a margin.  The limit is the context's and holds memory for every
+// resident thread of the device: the 12 KB that the multi-jump routine called here once needed were
+// 3.8 GB.
 static size_t query32_stack() {
-  size_t need = 4 * sizeof(JumpStep<float, D32>) + 2048;   // >= the cumulative frames reported by ptxas
+  size_t need = 1024;
   const void *ks[] = {(const void *)fwd32_kernel<0>, (const void *)fwd32_kernel<1>, (const void *)fwd32_kernel<2>,
                       (const void *)adj32_kernel<0>, (const void *)adj32_kernel<1>, (const void *)adj32_kernel<2>};
   for (const void *k : ks) {
