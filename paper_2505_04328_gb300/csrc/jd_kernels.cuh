@@ -1287,8 +1287,8 @@ template <typename R, int D>
 struct PreDraws {
   const uint32_t *w;   // [Nt][mloc] Poisson words
   const R *z;          // [Nt][D][mloc] sub-step 0 normals
-  const R *s;          // [Nt][1 + 2D][mloc] a step with exactly one (additive) jump: its
-                       // slot-0 draws (time fraction, unit size, next normals); else unset
+  const R *s;          // [Nt][1 + 2D][mloc] a step that takes the one-jump path: its slot-0
+                       // draws (time fraction, unit size, next normals); else unset
   Pair<R> *cw, *cw2;   // [mloc] each path's cost pair (first, second control)
   unsigned long long *held, key;   // the sweep records that the buffers hold the draws of key
 };
@@ -1362,6 +1362,7 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
                                          const JLog<R, D> &jl, int *__restrict__ jcnt, int64_t mloc,
                                          const PairOut<R, D> &p2, const PreDraws<R, D> &pd, Pair<R> *red,
                                          PreRing<R, D, DU> *ring = nullptr, SlotScratch<R, D> *slots = nullptr) {
+  static_assert(!(PRE && PAIR), "a pre-drawn pair runs as two single sweeps (fwd_kernel)");
   if (PRE && threadIdx.x >= SPREAD_LANES) return;   // no warp-wide operation follows in this mode
   const int64_t lm = PRE ? bid * SPREAD_LANES + threadIdx.x : bid * TPB + threadIdx.x;
   const bool active = lm < mloc;
@@ -1435,15 +1436,7 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
       const R *sk = pd.s + (int64_t)k * (1 + 2 * D) * mloc + lmc;
       if (has_jump(kp, w0) && one_jump(kp, w0)) {   // the common jump step, pre-drawn
         one_jump_pre(kp, k, sk, mloc, z, uk, x, lw);
-        if constexpr (PAIR) {
-          R uk2[DU];
-#pragma unroll
-          for (int l = 0; l < DU; ++l) uk2[l] = __ldg(p2.u + (size_t)k * DU + l);
-          one_jump_pre(kp, k, sk, mloc, z, uk2, x2, lw2);
-        }
         nj = 1;
-      } else if constexpr (PAIR) {
-        nj = forward_step2<R, D, DU, LW, KH, RK>(kp, kh, k, m, w0, z, u, x, lw, p2.u, x2, lw2);
       } else {
         nj = step_from_draws<R, D, DU, LW, true, KH, RK>(kp, kh, k, m, w0, z, uk, x, lw);
       }
@@ -1485,9 +1478,6 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
   if constexpr (PRE) {   // the path's pair; spread_combine_kernel sums them
     if (bid == 0 && threadIdx.x == 0) *pd.held = pd.key;   // the draws kernel has completed
     if (active) pd.cw[lm] = v;
-    if constexpr (PAIR) {
-      if (active) pd.cw2[lm] = cost2.pair();
-    }
   } else {
     const double s = block_sum_to_double(v, red);
     if (threadIdx.x == 0) partC[bid] = s;
@@ -1702,9 +1692,10 @@ fwd_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u
            uint32_t *__restrict__ flags, R *__restrict__ ckpt, R *__restrict__ pcost,
            JLog<R, D> jl, int *__restrict__ jcnt, int64_t mloc, PairOut<R, D> p2, PreDraws<R, D> pd = {}) {
   __shared__ Pair<R> red[TPB / 32];
-  // the round keys of kp in the draws: the paired, checkpoint and cost sweeps run faster
-  // with them; the single store sweep's register allocation did not (288.7 -> 298.4
-  // warp-instructions per warp-step, 9.75 -> 9.97 ms per launch at M = 2^20, N_t = 1000)
+  // the round keys of kp in the draws: the chunked sweeps always; step by step, the paired,
+  // checkpoint and cost sweeps run faster with them, the single store sweep's register allocation
+  // did not (d = 2, M = 2^20, N_t = 1000: 9.75 -> 9.97 ms per launch, 288.7 -> 298.4
+  // warp-instructions per warp-step)
   constexpr bool RK = !(MODE == FWD_STORE && !PAIR);
   if constexpr (PAIR && PRE) {
     // a pre-drawn pair: each control on its own warps (the first half of the blocks, then

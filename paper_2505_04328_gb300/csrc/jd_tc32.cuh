@@ -7,8 +7,9 @@
 // a BF16 high part and a BF16 low part and issues three products (hi*hi + hi*lo + lo*hi),
 // which keeps about 16 mantissa bits.  The adjoint's A^T lambda uses the same scheme.
 // Everything else (noise, jumps, cost, reductions) is the same FP32 arithmetic as the
-// generic kernels; steps with jumps run entirely on the CUDA cores through the generic
-// jump routines.
+// generic kernels; steps with jumps run entirely on the CUDA cores: in the forward by the whole
+// warp (coop_one_jumps, coop_jumps), in the adjoint from the jump log by the lane, with the CUDA
+// cores' products warp-wide (coop_adj_product).
 //
 // tcgen05 usage: warp 0 allocates 32 TMEM columns; every step all threads write their
 // row of the operand tile (K-major, no swizzle: 8-row x 16-byte core matrices, 128 B
@@ -445,8 +446,8 @@ __device__ __forceinline__ void coop_jumps(const KP32 &kp, const float *at, floa
   uint32_t *wu = reinterpret_cast<uint32_t *>(ws);
   auto mword = [&](int w) -> uint32_t & { return wu[(w >> 5) * TPB + (w & 31)]; };
   auto sword = [&](int w) -> uint32_t & { return wu[(2 + (w >> 5)) * TPB + (w & 31)]; };
-  float *zm = ws + 5 * TPB, *zs = ws + 6 * TPB, *zp = ws + 7 * TPB, *yv = ws + 8 * TPB, *xv = ws + 9 * TPB,
-        *ts = ws + 10 * TPB, *to = ws + 11 * TPB;
+  float *zm = ws + 5 * TPB, *zs = ws + 6 * TPB, *zp = ws + 7 * TPB, *yv = ws + 8 * TPB, *ts = ws + 10 * TPB,
+        *to = ws + 11 * TPB;
   int *ord = reinterpret_cast<int *>(ws + 12 * TPB);
   while (om) {
     const int j = __ffs((int)om) - 1;
