@@ -411,13 +411,14 @@ __device__ __forceinline__ void noisy_update(R de, const R (&f)[D], const R (&a)
 
 // Step k from x (in place) once the main-stream draws z and the Poisson word w0 are
 // taken; returns the number of jumps.
-// INLINE_JUMP: the one-jump case inline, or out of line (the replay of the parameter-
-// gradient recompute adjoint, whose loop must stay small for the instruction cache, and
-// the paired sweep of two controls).
+// ONE_JUMP: the one-jump case inline; out of line (the replay of the parameter-gradient recompute
+// adjoint, whose loop must stay small for the instruction cache); or not at all (the caller has
+// taken it: the paired sweep of two controls).
 // kh: the source of the drift, noise and step coefficients of the step without jumps
 // (kp itself or a HotFwd); the jump paths read kp.  RK: the inline slot draws take the
 // round keys of kp (a __grid_constant__ parameter).
-template <typename R, int D, int DU, typename LW, bool INLINE_JUMP = true, typename KH = KParams<R, D, DU>,
+enum OneJump { ONE_INLINE, ONE_CALL, ONE_TAKEN };
+template <typename R, int D, int DU, typename LW, OneJump ONE_JUMP = ONE_INLINE, typename KH = KParams<R, D, DU>,
           bool RK = false, bool COOP = false>
 __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, const KH &kh, int k, uint32_t m,
                                                uint32_t w0, const R (&z)[D], const R (&uk)[DU], R (&x)[D],
@@ -442,7 +443,7 @@ __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, cons
     plain_update(kh, f, z, x);
     return 0;
   }
-  if (!INLINE_JUMP && kp.jump_law != JD_JUMP_KS && one_jump(kp, w0)) {
+  if (ONE_JUMP == ONE_CALL && kp.jump_law != JD_JUMP_KS && one_jump(kp, w0)) {
     // copies: an address taken of x or uk themselves would move them to local memory
     R zc[D], xc[D], uc[DU], y1[D];
 #pragma unroll
@@ -460,7 +461,7 @@ __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, cons
     }
     return 1;
   }
-  if (!COOP && INLINE_JUMP && one_jump(kp, w0)) {
+  if (!COOP && ONE_JUMP == ONE_INLINE && one_jump(kp, w0)) {
     R xih[D], z1[D];
     const R th = slot0_draws<RK>(kp, k, m, xih, z1);
     one_jump_inline(kp, k, th, xih, z, z1, uk, x, lw);
@@ -496,7 +497,7 @@ __device__ __forceinline__ int step_from_draws(const KParams<R, D, DU> &kp, cons
 // One uniform step k from x (in place); returns the number of jumps.  With a LogWriter
 // the post-jump states of the step are recorded.  zo (optional, stride zs) receives the
 // step's main-stream normals Z_{k,0}.
-template <typename R, int D, int DU, typename LW, bool ZOUT = false, bool INLINE_JUMP = true,
+template <typename R, int D, int DU, typename LW, bool ZOUT = false, OneJump ONE_JUMP = ONE_INLINE,
           typename KH = KParams<R, D, DU>, bool RK = false, bool COOP = false>
 __device__ __forceinline__ int forward_step_h(const KParams<R, D, DU> &kp, const KH &kh, int k, uint32_t m,
                                               const R *__restrict__ u, R (&x)[D], LW &lw,
@@ -510,14 +511,14 @@ __device__ __forceinline__ int forward_step_h(const KParams<R, D, DU> &kp, const
   R uk[DU];
 #pragma unroll
   for (int l = 0; l < DU; ++l) uk[l] = __ldg(u + (size_t)k * DU + l);
-  return step_from_draws<R, D, DU, LW, INLINE_JUMP, KH, RK, COOP>(kp, kh, k, m, w0, z, uk, x, lw, sc);
+  return step_from_draws<R, D, DU, LW, ONE_JUMP, KH, RK, COOP>(kp, kh, k, m, w0, z, uk, x, lw, sc);
 }
 
-template <typename R, int D, int DU, typename LW, bool ZOUT = false, bool INLINE_JUMP = true, bool COOP = false>
+template <typename R, int D, int DU, typename LW, bool ZOUT = false, OneJump ONE_JUMP = ONE_INLINE, bool COOP = false>
 __device__ __forceinline__ int forward_step(const KParams<R, D, DU> &kp, int k, uint32_t m,
                                             const R *__restrict__ u, R (&x)[D], LW &lw,
                                             R *zo = nullptr, int zs = 0, SlotScratch<R, D> *sc = nullptr) {
-  return forward_step_h<R, D, DU, LW, ZOUT, INLINE_JUMP, KParams<R, D, DU>, false, COOP>(kp, kp, k, m, u, x, lw, zo,
+  return forward_step_h<R, D, DU, LW, ZOUT, ONE_JUMP, KParams<R, D, DU>, false, COOP>(kp, kp, k, m, u, x, lw, zo,
                                                                                         zs, sc);
 }
 
@@ -550,8 +551,8 @@ __device__ __forceinline__ int forward_step2(const KParams<R, D, DU> &kp, const 
     one_jump_inline(kp, k, th, xih, z, z1, uk2, x2, lw2);
     return 1;
   }
-  const int n = step_from_draws<R, D, DU, LW, false>(kp, kp, k, m, w0, z, uk, x, lw);
-  step_from_draws<R, D, DU, LW, false>(kp, kp, k, m, w0, z, uk2, x2, lw2);
+  const int n = step_from_draws<R, D, DU, LW, ONE_TAKEN>(kp, kp, k, m, w0, z, uk, x, lw);
+  step_from_draws<R, D, DU, LW, ONE_TAKEN>(kp, kp, k, m, w0, z, uk2, x2, lw2);
   return n;
 }
 
@@ -1438,14 +1439,14 @@ __device__ __forceinline__ void fwd_body(const KParams<R, D, DU> &kp, int64_t bi
         one_jump_pre(kp, k, sk, mloc, z, uk, x, lw);
         nj = 1;
       } else {
-        nj = step_from_draws<R, D, DU, LW, true, KH, RK>(kp, kh, k, m, w0, z, uk, x, lw);
+        nj = step_from_draws<R, D, DU, LW, ONE_INLINE, KH, RK>(kp, kh, k, m, w0, z, uk, x, lw);
       }
     } else if constexpr (PAIR) {
       R z[D];
       const uint32_t w0 = main_draws<RK>(kp, k, m, z);
       nj = forward_step2<R, D, DU, LW, KH, RK>(kp, kh, k, m, w0, z, u, x, lw, p2.u, x2, lw2);
     } else {
-      nj = forward_step_h<R, D, DU, LW, false, true, KH, RK, COOP>(kp, kh, k, m, u, x, lw, nullptr, 0, slots);
+      nj = forward_step_h<R, D, DU, LW, false, ONE_INLINE, KH, RK, COOP>(kp, kh, k, m, u, x, lw, nullptr, 0, slots);
     }
     if (nj) fw |= 1u << (k & 31);
     if constexpr (PRE)
@@ -2127,7 +2128,7 @@ __device__ __forceinline__ void adj_recompute_body(const KParams<R, D, DU> &kp, 
       for (int i = 0; i < len; ++i) {
   #pragma unroll
         for (int c = 0; c < D; ++c) sbuf[(i * D + c) * TPB + tid] = x[c];
-        if (forward_step<R, D, DU, LWR, ZBUF, !THETA, (D > 2 && RCH)>(
+        if (forward_step<R, D, DU, LWR, ZBUF, THETA ? ONE_CALL : ONE_INLINE, (D > 2 && RCH)>(
                 kp, k0 + i, m, u, x, lw, zbuf + (size_t)i * D * TPB + tid, TPB, slots))
           jm |= 1ull << i;
       }

@@ -106,7 +106,7 @@ inline bool coop_slots(const FormKey &f, SweepKind kind) {
 inline bool chunk_steps(const FormKey &f, SweepKind kind) {
   double lo = 0.0, hi = 0.5;
   if (f.f64) {
-    if (f.D == 2) hi = 0.3;
+    if (f.D == 2) hi = f.ks ? 0.45 : 0.3;   // Keilson-Storer at 0.4 5.27 -> 5.12
     if (f.ks && kind != SWEEP_REPLAY) lo = 0.004;
   } else {
     if (f.D == 2 && kind == SWEEP_REPLAY && f.M > 152 * 5 * 128) hi = 0.08;

@@ -158,6 +158,8 @@ CHUNKS = [
     (2, True, KS, STORE, 0.0, False),           # 0.71 -> 0.79
     (2, True, KS, PAIR, 0.003, False),          # 1.17 -> 1.25
     (2, True, KS, STORE, 0.006, True),          # 1.04 -> 0.96
+    (2, True, KS, COST, 0.4, True),             # 5.27 -> 5.12
+    (2, True, KS, PAIR, 0.6, False),            # 10.8 -> 12.0
     (2, True, UNIFORM, STORE, 0.0, True),       # 0.81 -> 0.79
     (1, False, NORMAL, COST, 0.002, False),    # 0.945 -> 0.977
     (1, False, NORMAL, COST, 0.008, True),     # 1.20 -> 1.13
