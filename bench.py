@@ -1007,12 +1007,12 @@ COUNTERS = {
     # M = 2^20 over N_t = 100 steps of the workload's step length; the d = 32 kernels in
     # BF16 tensor-core mode at M = 2^16 (512 tiles), N_t = 100 steps of theirs.  All in
     # profiles/counters_path_kernels.md
-    ("double_well", "fwd_pair"): ("5dc9d63a7146", 17.87, 309.1),
-    ("double_well", "fwd_store"): ("5dc9d63a7146", 8.66, 241.7),
-    ("double_well", "adj_stored"): ("5dc9d63a7146", 8.79, 60.2),
-    ("double_well", "adj_recompute"): ("5dc9d63a7146", 0.69, 300.6),
-    ("linear32/tc1", "fwd_store"): ("5dc9d63a7146", 123.2, 1930.4),
-    ("linear32/tc1", "adj_stored"): ("5dc9d63a7146", 139.7, 662.2),
+    ("double_well", "fwd_pair"): ("fcc322ef5b02", 17.87, 309.1),
+    ("double_well", "fwd_store"): ("fcc322ef5b02", 8.66, 241.7),
+    ("double_well", "adj_stored"): ("fcc322ef5b02", 8.79, 60.2),
+    ("double_well", "adj_recompute"): ("fcc322ef5b02", 0.69, 300.6),
+    ("linear32/tc1", "fwd_store"): ("fcc322ef5b02", 123.2, 1930.4),
+    ("linear32/tc1", "adj_stored"): ("fcc322ef5b02", 139.7, 662.2),
 }
 
 

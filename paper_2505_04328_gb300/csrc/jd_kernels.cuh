@@ -1976,8 +1976,17 @@ __device__ __forceinline__ void stored_sweep(const KParams<R, D, DU> &kp, const 
   finish_theta<R, D, DU, THETA>(kp, th, active, partT, red1, bid);
 }
 
+// Resident blocks asked of the compiler: its own choice for FP64, d <= 2 took 72 to 96 registers
+// and spilled 16 to 104 bytes; 96 for five blocks spill nothing.  N_t = 160, lambda dt = 0.2, d = 1:
+// M = 2^17 1.26 -> 1.11 ms, with parameter gradients 22.6 -> 20.2; M = 1000 0.239 -> 0.218 and 3.88
+// -> 3.31; d = 2 as before, with parameter gradients at 0.02 10.1 -> 9.33 (2^17).
+template <typename R, int D>
+constexpr int adj_stored_blocks() {
+  return sizeof(R) == 8 && D <= 2 ? 5 : 0;
+}
+
 template <typename R, int D, int DU, bool THETA, bool LAM = false>
-__global__ void __launch_bounds__(TPB)
+__global__ void __launch_bounds__(TPB, adj_stored_blocks<R, D>())
 adj_stored_kernel(const __grid_constant__ KParams<R, D, DU> kp, const R *__restrict__ u,
                   const R *__restrict__ xd, const R *__restrict__ traj,
                   const uint32_t *__restrict__ flags, JLog<R, D> jl, const int *__restrict__ jcnt,
