@@ -84,7 +84,8 @@ inline bool coop_slots(const FormKey &f, SweepKind kind) {
 // d <= 2: whether a sweep takes its steps in chunks, by the jump rate per step.  The chunks'
 // passes cost a little where almost nothing jumps, and at high rates most jump steps have three
 // jumps or more and go to the general routine either way.  One launch at N_t = 160, step by
-// step -> in chunks, in ms (FP32 M = 2^18, the rates up to 0.01 of d = 1 and 2 at 2^20; FP64 2^15):
+// step -> in chunks, in ms (pair: checkpoints; FP32 M = 2^18, but 2^20 up to 0.006, pairs up to
+// 0.002; FP64 2^15):
 //   lambda dt              0             0.002         0.006         0.1           0.3           0.5           0.6
 //   FP32 d = 1  cost       0.85 -> 0.85  0.95 -> 0.98  1.12 -> 1.09  0.96 -> 0.62  2.32 -> 1.30  3.12 -> 2.52  3.37 -> 3.10
 //               ckpt.      0.83 -> 0.88  0.93 -> 1.00  1.10 -> 1.11  0.95 -> 0.63  2.34 -> 1.31  3.16 -> 2.50  3.42 -> 3.09
