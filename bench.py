@@ -1007,12 +1007,12 @@ COUNTERS = {
     # M = 2^20 over N_t = 100 steps of the workload's step length; the d = 32 kernels in
     # BF16 tensor-core mode at M = 2^16 (512 tiles), N_t = 100 steps of theirs.  All in
     # profiles/counters_path_kernels.md
-    ("double_well", "fwd_pair"): ("8b5d685d1153", 17.87, 309.1),
-    ("double_well", "fwd_store"): ("8b5d685d1153", 8.66, 241.7),
-    ("double_well", "adj_stored"): ("8b5d685d1153", 8.79, 60.2),
-    ("double_well", "adj_recompute"): ("8b5d685d1153", 0.69, 300.6),
-    ("linear32/tc1", "fwd_store"): ("8b5d685d1153", 123.2, 1930.4),
-    ("linear32/tc1", "adj_stored"): ("8b5d685d1153", 139.7, 662.2),
+    ("double_well", "fwd_pair"): ("1f3aa80afb24", 17.87, 309.1),
+    ("double_well", "fwd_store"): ("1f3aa80afb24", 8.66, 241.7),
+    ("double_well", "adj_stored"): ("1f3aa80afb24", 8.79, 60.2),
+    ("double_well", "adj_recompute"): ("1f3aa80afb24", 0.69, 300.6),
+    ("linear32/tc1", "fwd_store"): ("1f3aa80afb24", 123.2, 1930.4),
+    ("linear32/tc1", "adj_stored"): ("1f3aa80afb24", 139.7, 662.2),
 }
 
 

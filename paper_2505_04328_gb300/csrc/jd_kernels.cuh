@@ -261,12 +261,18 @@ __host__ __device__ constexpr int seg_len() {
 // the additive laws for larger d (whose sweeps ran 1% slower with the law's branch).
 template <int D>
 constexpr bool ONE_JUMP_KS = D <= 2;
-// A step with jumps has exactly one, and the problem's steps take the one-jump paths (make_kparams;
-// a test of the law here beside that of the words cost the pre-drawn sweeps, whose steps are one
-// chain, 5%: d = 1 pair, M = 1000, N_t = 200, FP32, lambda dt = 0.07: 103 against 98 us).
+// A step with jumps has exactly one, and the problem's steps take the one-jump paths (make_kparams:
+// one_jump_path).  For d <= 2 one field says so: a test of the law here beside that of the words cost
+// the pre-drawn sweeps, whose steps are one chain, 5% (d = 1 pair, M = 1000, N_t = 200, FP32, lambda
+// dt = 0.07: 103 against 98 us).  For d > 2, where the field would say the same, the two tests leave
+// the better register allocation: d = 3 gradient, M = 19,977, N_t = 541, lambda dt = 0.005, FP32, 599
+// against 607 us.
 template <typename R, int D, int DU>
 __device__ __forceinline__ bool one_jump(const KParams<R, D, DU> &kp, uint32_t w0) {
-  return kp.one_pairs == MainWords<D>::PD && (unsigned long long)w0 < kp.thr[1];
+  if constexpr (D > 2)
+    return kp.jump_law != JD_JUMP_KS && kp.npair == MainWords<D>::PD && (unsigned long long)w0 < kp.thr[1];
+  else
+    return kp.one_pairs == MainWords<D>::PD && (unsigned long long)w0 < kp.thr[1];
 }
 
 // The jump of a one-jump step (apply_jump; the additive map without its product by jgain = 1,
