@@ -600,6 +600,21 @@ static size_t base_bytes(const jd_problem_desc &q, int D, int DU, size_t es) {
          (D == 32 ? 16384 + (size_t)q.Nt * 32 * sizeof(float) : 0);
 }
 
+// Whether a small problem gets the pre-pass buffers.  Up to 6080 paths, where some sweep takes them
+// at the present jump rate, they are part of the memory that the problem needs; beyond, or where
+// only an update could ask for them, the budget has to hold them beside the plan that the problem
+// has without them.
+static bool keep_pre(const jd_problem_desc &q, int D, int DU, size_t es, size_t budget) {
+  if (!pre_pass(q, D, es)) return false;
+  const FormKey form = form_key(D, es == 8, q);
+  int64_t now = 0;
+  for (int kind = SWEEP_COST; kind < SWEEP_REPLAY; ++kind)
+    now = std::max(now, pre_max_paths(form, (SweepKind)kind));
+  if (q.M <= std::min<int64_t>(now, 152 * 40)) return true;
+  const size_t plan = q.mode == JD_ADJ_RECOMPUTE ? ckpt_bytes(q, D, es, 16) : stored_plan_bytes(q, D, es, q.M);
+  return base_bytes(q, D, DU, es) + plan <= budget;
+}
+
 // Allocate the trajectory or checkpoint buffers on first use.
 static jd_status ensure_plan(jd_problem *p) {
   if (p->plan != JD_ADJ_AUTO) return JD_OK;
@@ -1577,7 +1592,7 @@ jd_status jd::create_problem(const jd_problem_desc &q, const jd::ProblemOpts &op
   ALLOC(p->partG, (size_t)q.Nt * p->DU * grad_parts(q.M) * 8, "gradient partials");
   ALLOC(p->partT, (size_t)(p->D + 2) * p->nblk * 8, "parameter partials");
   ALLOC(p->units, (size_t)n_units(q.M) * (1 + nu) * 8, "unit sums");
-  if (!opts.no_pre && pre_pass(q, p->D, es)) {   // a small problem: the draws' pre-pass buffers
+  if (!opts.no_pre && keep_pre(q, p->D, p->DU, es, p->budget)) {   // a small problem: the draws' pre-pass buffers
     ALLOC(p->pre_w, (size_t)q.Nt * q.M * 4, "pre-drawn Poisson words");
     ALLOC(p->pre_z, pre_z_values(q.Nt, p->D, q.M) * es, "pre-drawn normals and slot draws");
     ALLOC(p->pre_key, sizeof(unsigned long long), "pre-drawn key");

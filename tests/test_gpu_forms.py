@@ -127,3 +127,26 @@ def test_feedback_fp64_sizes_and_rings(nx, particles):
         J, g = jp.fb_gradient(fb, mu)
         assert jp.fb_cost(fb, mu) == J
     assert abs(J - Jo) <= 1e-13 * abs(Jo) and np.linalg.norm(g - go) <= 1e-12 * np.linalg.norm(go)
+
+
+@pytest.mark.parametrize("mode,plan", [("auto", "stored"), ("stored", "stored"), ("recompute", "recompute")])
+def test_pre_pass_buffers_give_way_to_a_small_budget(mode, plan):
+    """A problem that only a higher jump rate would pre-draw runs in the memory that it needs
+    without the buffers, in the plan that it has without them."""
+    M, Nt = 8000, 400
+    p = workloads.lq_scalar(M=M, Nt=Nt)
+    low, high = p.replace(lam=0.002 * Nt), p.replace(lam=0.1 * Nt)
+    u = workloads.random_control(p, seed=3, scale=0.6)
+    buffers = Nt * M * 4 + (Nt * 4 * M + 4 * M) * 4 + 8
+    with JdProblem(low, mode=mode) as jp:
+        J, g, _ = jp.gradient(u)
+        full = jp.info()["device_bytes"]
+    with JdProblem(low, mode=mode, mem_budget=full - buffers) as jp:
+        assert jp.info()["device_bytes"] < full - buffers
+        J1, g1, _ = jp.gradient(u)
+        assert jp.info() == dict(device_bytes=full - buffers, mode=plan)
+        jp.update(high)
+        J2, n2 = _launches(lambda: jp.cost(u))
+    with JdProblem(high, mode=mode) as jp:
+        J3, n3 = _launches(lambda: jp.cost(u))
+    assert J1 == J and np.array_equal(g1, g) and J2 == J3 and n3 == n2 + PRE_EXTRA
